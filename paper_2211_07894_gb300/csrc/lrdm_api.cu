@@ -818,6 +818,7 @@ lrdm_status create_ctx(lrdm_ctx** out, const lrdm_system* sys, int nsys, const l
     if ((rc = dalloc(ctx, &ctx->d_round, 1)) != LRDM_OK) break;
     const int maxval = KMAX_LIMIT * (KMAX_LIMIT + 1) / 2 + KMAX_LIMIT + 1;
     if ((rc = dalloc(ctx, &ctx->ls_partial, (size_t)LS_BLOCKS * maxval)) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->ls_sums, maxval)) != LRDM_OK) break;
     if ((rc = dalloc(ctx, &ctx->ls_coef, KMAX_LIMIT)) != LRDM_OK) break;
     if ((rc = dalloc(ctx, &ctx->ls_scal, 4)) != LRDM_OK) break;
     if ((rc = dalloc(ctx, &ctx->upd_partial, UPD_BLOCKS)) != LRDM_OK) break;
@@ -936,11 +937,11 @@ lrdm_status lrdm_apply(lrdm_ctx* ctx, int sys, const void* R, const void* v, con
   if (!isfinite(alpha)) return LRDM_ERR_INVALID_ARG;
   SysState& S = ctx->sys[sys];
   long long n = (long long)S.nspin * S.Ng;
-  count(ctx, 4);
+  count(ctx, 5);
   int ar_failed = 0;
   const lrdm_status rc = from_cuda(launch_ls(R, v, f, ctx->opt.io_dtype, K, n, S.w, alpha,
                                              ctx->opt.pinv_rcond, rho_inout, ctx->ls_coef, coeff_out,
-                                             s_rel_out, ctx->ls_partial, ctx->ls_scal, ctx->upd_partial,
+                                             s_rel_out, ctx->ls_partial, ctx->ls_sums, ctx->ls_scal, ctx->upd_partial,
                                              ctx->d_status, static_cast<cudaStream_t>(stream),
                                              ctx->rows ? &ctx->ar : nullptr, &ar_failed));
   return ar_failed ? LRDM_ERR_COLLECTIVE : rc;
@@ -983,10 +984,10 @@ lrdm_status lrdm_krylov_step(lrdm_ctx* ctx, int sys, const void* R, double s_tol
     rank = i + 1;
     // least squares on the first i + 1 directions (no update yet) -> s_rel
     LRDM_CU(launch_ls(R, U, T, io, rank, n, S.w, 0.0, ctx->opt.pinv_rcond, nullptr, ctx->ls_coef,
-                      coeff_out, nullptr, ctx->ls_partial, ctx->ls_scal, ctx->upd_partial,
+                      coeff_out, nullptr, ctx->ls_partial, ctx->ls_sums, ctx->ls_scal, ctx->upd_partial,
                       ctx->d_status, st, ar, &ar_failed));
     if (ar_failed) return LRDM_ERR_COLLECTIVE;
-    count(ctx, 4);
+    count(ctx, 5);
     double s_rel = 0.0;
     LRDM_CU(cudaMemcpyAsync(&s_rel, ctx->ls_scal + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
     LRDM_CU(cudaStreamSynchronize(st));
@@ -1003,10 +1004,10 @@ lrdm_status lrdm_krylov_step(lrdm_ctx* ctx, int sys, const void* R, double s_tol
   if (rho_inout) {
     const double a = alpha < 0.0 ? (r_norm < 2.0 ? 0.5 : 0.1) : alpha;
     LRDM_CU(launch_ls(R, U, T, io, rank, n, S.w, a, ctx->opt.pinv_rcond, rho_inout, ctx->ls_coef,
-                      coeff_out, nullptr, ctx->ls_partial, ctx->ls_scal, ctx->upd_partial,
+                      coeff_out, nullptr, ctx->ls_partial, ctx->ls_sums, ctx->ls_scal, ctx->upd_partial,
                       ctx->d_status, st, ar, &ar_failed));
     if (ar_failed) return LRDM_ERR_COLLECTIVE;
-    count(ctx, 4);
+    count(ctx, 5);
   }
   return LRDM_OK;
 }

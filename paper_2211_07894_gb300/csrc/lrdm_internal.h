@@ -138,6 +138,7 @@ struct lrdm_ctx {
   int* d_status = nullptr;
   unsigned* d_round = nullptr;       // round counter of the tensor-core contractions (zeroed per launch)
   double* ls_partial = nullptr;      // [LS_BLOCKS][max values]
+  double* ls_sums = nullptr;         // [max values] Gram sums over the blocks
   double* ls_coef = nullptr;         // [KMAX_LIMIT]
   double* ls_scal = nullptr;         // [4]: r2, s_rel scratch
   double* upd_partial = nullptr;     // [UPD_BLOCKS]
@@ -321,7 +322,7 @@ cudaError_t launch_norm(const void* x, int io, long long n, double w, double* sc
 cudaError_t launch_ls(const void* R, const void* v, const void* f, int io_dtype, int K,
                       long long n, double w, double alpha, double rcond, void* rho_inout,
                       double* coef, double* coeff_out, double* s_rel_out, double* partial,
-                      double* scal, double* upd_partial, int* status, cudaStream_t st,
+                      double* sums, double* scal, double* upd_partial, int* status, cudaStream_t st,
                       const AllReduce* ar = nullptr, int* ar_failed = nullptr);
 
 // allocation-free least-squares step (k_ls.cu, static device scratch)

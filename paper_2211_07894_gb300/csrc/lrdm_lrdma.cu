@@ -27,6 +27,7 @@ struct lrdm_lrdma {
   double* gs = nullptr;              // Gram-Schmidt / norm scratch
   double* norm = nullptr;            // [2]
   double* ls_partial = nullptr;
+  double* ls_sums = nullptr;
   double* ls_coef = nullptr;
   double* ls_scal = nullptr;
   double* upd_partial = nullptr;
@@ -59,7 +60,7 @@ lrdm_status lrdma_ls(lrdm_lrdma* a, const void* R, const void* v, int m, double 
                      double rcond, double* s_rel, cudaStream_t st, const AllReduce* ar) {
   int ar_failed = 0;
   LRDM_CU(launch_ls(R, v, a->T, a->io, m, a->n, a->w, alpha, rcond, rho, a->ls_coef, nullptr,
-                    nullptr, a->ls_partial, a->ls_scal, a->upd_partial, a->status, st, ar,
+                    nullptr, a->ls_partial, a->ls_sums, a->ls_scal, a->upd_partial, a->status, st, ar,
                     &ar_failed));
   if (ar_failed) return LRDM_ERR_COLLECTIVE;
   LRDM_CU(cudaMemcpyAsync(s_rel, a->ls_scal + 1, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -105,6 +106,7 @@ lrdm_status lrdm_lrdma_create(lrdm_lrdma** out, long long n, int io_dtype, doubl
       (rc = lalloc(a, &a->gs, gram_schmidt_scratch())) != LRDM_OK ||
       (rc = lalloc(a, &a->norm, 2)) != LRDM_OK ||
       (rc = lalloc(a, &a->ls_partial, (size_t)LS_BLOCKS * maxval)) != LRDM_OK ||
+      (rc = lalloc(a, &a->ls_sums, maxval)) != LRDM_OK ||
       (rc = lalloc(a, &a->ls_coef, KMAX_LIMIT)) != LRDM_OK ||
       (rc = lalloc(a, &a->ls_scal, 4)) != LRDM_OK ||
       (rc = lalloc(a, &a->upd_partial, UPD_BLOCKS)) != LRDM_OK ||
