@@ -492,6 +492,30 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // acc-full barriers; the epilogue warps of both CTAs arrive on the even CTA's
 // acc-empty barrier (8 arrivals).  Items: as k_gemm2_tc with P.nR = the
 // number of 256-row blocks.
+//
+// Only the triangle is multiplied: X'' is zero below its diagonal, so in the
+// tile's diagonal block a stage of 32 states i0 .. needs the columns j >= i0
+// alone, and past the last state there is nothing.  A stage's MMAs run at
+// N = its columns (a multiple of 32, from 256 down to 32) into the
+// accumulator's last N columns; CTA r loads N / 2 X'' rows (one box of 64 rows
+// or of 128: the rate at which boxes are issued counts, boxes of 32 rows took
+// 546 against 475 us in TF32 at 48^3 / 512).  Against full 256-wide blocks
+// that is 0.49 of the MMA work at N_s = 384, 0.71 at 512, 0.86 at 1024 and 0.97
+// at 4096, and N_s is not rounded up to 128 or 256.
+//
+// The row-dot reads Psi(rows, J) through shared memory: chunks of 32 states,
+// loaded by TMA (warp 6) into a ring of two and read back one row a thread
+// without bank conflicts.  Loaded straight from global memory, a row a
+// thread, each 16-byte load touched 32 lines, 8,192 L1 wavefronts a tile and
+// more than the MMAs of a narrow subspace take (L1 71 % busy, tensor pipe
+// idle half the time at N_s = 512).
+//
+// Both together on one GB300, before -> now: 48^3 / 512, K = 8: 633 -> 515 us
+// (TF32 582 -> 474), K = 1: 104 -> 85 us; 64^3 / 1024, K = 16: 8.9 -> 8.2 ms;
+// 72^3 / 2048, K = 12: 33.2 -> 32.5 ms; 96^3 / 4096, K = 16: 394 -> 387 ms.
+// What is left at small N_s is the operand feed: L2 delivers 8 to 13 TB/s to
+// the SMs (31 B per clock and SM from 60 MB, TMA alone), a stage of 32 KB in
+// 700 to 900 clocks against 768 of MMAs at N = 256 and fewer in the triangle.
 
 template <int PREC>
 struct G2PCfg {
@@ -502,13 +526,60 @@ struct G2PCfg {
   static constexpr int CHUNK = PARTS * (TILE_A + TILE_B);
   static constexpr int SB = SUB * CHUNK;
   static constexpr int STAGES = 6;
-  static constexpr int SMEM = STAGES * SB + 1024 + 512;
-  static constexpr uint32_t IDESC = ptx::idesc_make(PREC == LRDM_BF16X3 ? 1 : 2, 256, 256);
+  static constexpr int ESB = 2 * TILE_A;                // Psi(rows, 32 states) of the row-dot: hi and lo, or two TF32 chunks
+  static constexpr int ESTAGES = 2;
+  static constexpr int E_OFF = STAGES * SB;
+  static constexpr int SMEM = E_OFF + ESTAGES * ESB + 1024 + 512;
+  static constexpr int THREADS = NTHREADS + 32;         // warp 6: TMA of the row-dot's Psi chunks
+  static constexpr uint32_t IDESC = ptx::idesc_make(PREC == LRDM_BF16X3 ? 1 : 2, 256, 0);   // N per stage
   static_assert(SMEM <= 227 * 1024, "shared memory budget");
+  static_assert(BK * SUB == 32, "a stage holds 32 states");
 };
 
+// Row-dot of 32 columns (v, from tensor memory) with a thread's Psi row chunk
+// at shared address sp (64-byte rows, 64-byte swizzle; BF16x3: hi, lo 8 KB
+// further; TF32: states 0-15, 16-31 8 KB further), in ascending states.
 template <int PREC>
-__device__ __forceinline__ void issue_g2p_mmas(uint32_t d, uint32_t sa, uint32_t first) {
+__device__ __forceinline__ float g2p_dot(float part, const float (&v)[32], uint32_t sp, int row) {
+  const uint32_t ra = sp + row * ROWB;
+  const int sw = (row >> 1) & 3;
+  uint4 w[8];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    w[u] = ptx::lds128(ra + ((u ^ sw) << 4));
+    w[4 + u] = ptx::lds128(ra + TILE_A + ((u ^ sw) << 4));
+  }
+  if (PREC == LRDM_BF16X3) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t hw[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+      const uint32_t lw[4] = {w[4 + u].x, w[4 + u].y, w[4 + u].z, w[4 + u].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        part += v[u * 8 + 2 * e] * (bf_lo(hw[e]) + bf_lo(lw[e]));
+        part += v[u * 8 + 2 * e + 1] * (bf_hi(hw[e]) + bf_hi(lw[e]));
+      }
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      part += v[u * 4] * __uint_as_float(w[u].x) + v[u * 4 + 1] * __uint_as_float(w[u].y) +
+              v[u * 4 + 2] * __uint_as_float(w[u].z) + v[u * 4 + 3] * __uint_as_float(w[u].w);
+  }
+  return part;
+}
+
+// States of a problem that are multiplied, the columns of j-tile J and its
+// stages (32 states each), and the columns of stage ic.
+__device__ __forceinline__ int g2p_ns(const TcProblem* pr) { return (pr->ns + 31) & ~31; }
+__device__ __forceinline__ int g2p_cols(int ns, int J) { return min(256, ns - 256 * J); }
+__device__ __forceinline__ int g2p_stages(int ns, int J) { return min(256 * (J + 1), ns) / 32; }
+__device__ __forceinline__ int g2p_stage_cols(int ns, int J, int ic) {
+  return g2p_cols(ns, J) - max(0, 32 * ic - 256 * J);
+}
+
+template <int PREC>
+__device__ __forceinline__ void issue_g2p_mmas(uint32_t d, uint32_t sa, uint32_t idesc, uint32_t first) {
   using C = G2PCfg<PREC>;
   constexpr int PARTS = Tr<PREC>::PARTS;
   const uint32_t a0 = sa, a1 = sa + TILE_A;
@@ -518,24 +589,27 @@ __device__ __forceinline__ void issue_g2p_mmas(uint32_t d, uint32_t sa, uint32_t
     const uint32_t off = kk * 32;
     const uint32_t acc = (first && kk == 0) ? 0u : 1u;
     if (PREC == LRDM_BF16X3) {
-      ptx::mma_f16_pair(d, ptx::desc_k_sw64(a0 + off), ptx::desc_k_sw64(b0 + off), C::IDESC, acc);
-      ptx::mma_f16_pair(d, ptx::desc_k_sw64(a0 + off), ptx::desc_k_sw64(b1 + off), C::IDESC, 1);
-      ptx::mma_f16_pair(d, ptx::desc_k_sw64(a1 + off), ptx::desc_k_sw64(b0 + off), C::IDESC, 1);
+      ptx::mma_f16_pair(d, ptx::desc_k_sw64(a0 + off), ptx::desc_k_sw64(b0 + off), idesc, acc);
+      ptx::mma_f16_pair(d, ptx::desc_k_sw64(a0 + off), ptx::desc_k_sw64(b1 + off), idesc, 1);
+      ptx::mma_f16_pair(d, ptx::desc_k_sw64(a1 + off), ptx::desc_k_sw64(b0 + off), idesc, 1);
     } else {
-      ptx::mma_tf32_pair(d, ptx::desc_k_sw64(a0 + off), ptx::desc_k_sw64(b0 + off), C::IDESC, acc);
+      ptx::mma_tf32_pair(d, ptx::desc_k_sw64(a0 + off), ptx::desc_k_sw64(b0 + off), idesc, acc);
     }
   }
 }
 
 // Launched in clusters of two CTAs.
 template <int PREC>
-__global__ void __launch_bounds__(NTHREADS, 1)
+__global__ void __launch_bounds__(G2PCfg<PREC>::THREADS, 1)
     k_gemm2_pair(const __grid_constant__ G2Params P) {
   using C = G2PCfg<PREC>;
   constexpr int STAGES = C::STAGES, PARTS = C::PARTS, BK = C::BK, SB = C::SB, BN2 = C::BN2;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const Bars B = carve<STAGES>(smem + STAGES * SB);   // ready[] serves as the relayed full barrier
+  uint8_t* const tail = smem + C::E_OFF + C::ESTAGES * C::ESB;
+  const Bars B = carve<STAGES>(tail);                 // ready[] serves as the relayed full barrier
+  uint64_t* const efull = reinterpret_cast<uint64_t*>(tail) + 3 * STAGES + 8;    // row-dot chunk landed
+  uint64_t* const eempty = efull + C::ESTAGES;                                   // read by the four warps
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int items = P.begin[P.nslot];
   const int rank = (int)ptx::cluster_ctarank();
@@ -550,6 +624,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int a = 0; a < 2; ++a) {
       ptx::mbar_init(&B.acc_full[a], 1);
       ptx::mbar_init(&B.acc_empty[a], 8);
+    }
+    for (int a = 0; a < C::ESTAGES; ++a) {
+      ptx::mbar_init(&efull[a], 1);
+      ptx::mbar_init(&eempty[a], 4);
     }
     ptx::mbar_init(B.drain, 1);
     *B.abort = 0;
@@ -575,7 +653,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (PARTS == 2) {
         ptx::tmap_acquire(&pr->g2a1);
         ptx::tmap_acquire(&pr->g2b1);
+        ptx::tmap_acquire(&pr->g2c1);
       }
+      ptx::tmap_acquire(&pr->g2c0);
     }
     int s = 0;
     uint32_t ph = 0;
@@ -589,25 +669,29 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         align = false;
       int q, k, R2, jp, j0, j1;
       const TcProblem* pr = g2_item<BN2>(P, item, q, k, R2, jp, j0, j1);
-      const int ns_pad = pr->ns_pad;
+      const int ns = g2p_ns(pr);
       const int rb = 2 * R2 + rank;                       // this CTA's 128-row block (past the end: zero fill)
       bool ok = true;
       for (int jj = j0; jj < j1 && ok; ++jj) {
         const int J = g2_tile(P, q, jj);
-        const int nch = min((J + 1) * BN2, ns_pad) / (BK * C::SUB);
+        const int nch = g2p_stages(ns, J);
         for (int ic = 0; ic < nch; ++ic) {
           if (!wait1(&B.empty[s], ph ^ 1, B, P.status)) { ok = false; break; }
-          ptx::mbar_arrive_expect_tx(&B.full[s], SB);
+          const int n = g2p_stage_cols(ns, J, ic);
+          // this CTA's half of the stage's columns: the last n of the tile
+          const int jr = J * BN2 + g2p_cols(ns, J) - n + rank * (n / 2);
+          const bool half = n <= 128;                         // 64 X'' rows suffice
+          ptx::mbar_arrive_expect_tx(&B.full[s], C::SUB * PARTS * (TILE_A + (half ? C::TILE_B / 2 : C::TILE_B)));
 #pragma unroll
           for (int c = 0; c < C::SUB; ++c) {
             uint8_t* st = smem + s * SB + c * C::CHUNK;
             const int i0 = (ic * C::SUB + c) * BK;
             ptx::tma_load_2d(st, &pr->g2a0, &B.full[s], i0, rb * BM);
             if (PARTS == 2) ptx::tma_load_2d(st + TILE_A, &pr->g2a1, &B.full[s], i0, rb * BM);
-            ptx::tma_load_3d(st + PARTS * TILE_A, &pr->g2b0, &B.full[s], i0, J * BN2 + rank * 128, k);
+            uint8_t* sb = st + PARTS * TILE_A;
+            ptx::tma_load_3d(sb, half ? &pr->g2c0 : &pr->g2b0, &B.full[s], i0, jr, k);
             if (PARTS == 2)
-              ptx::tma_load_3d(st + PARTS * TILE_A + C::TILE_B, &pr->g2b1, &B.full[s], i0,
-                               J * BN2 + rank * 128, k);
+              ptx::tma_load_3d(sb + C::TILE_B, half ? &pr->g2c1 : &pr->g2b1, &B.full[s], i0, jr, k);
           }
           pending[s] = (int)ph;
           if (++s == STAGES) { s = 0; ph ^= 1; }
@@ -626,22 +710,25 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int item = pair; item < items && ok; item += npairs) {
       int q, k, R2, jp, j0, j1;
       const TcProblem* pr = g2_item<BN2>(P, item, q, k, R2, jp, j0, j1);
-      const int ns_pad = pr->ns_pad;
+      const int ns = g2p_ns(pr);
       for (int jj = j0; jj < j1 && ok; ++jj) {
         const int J = g2_tile(P, q, jj);
         if (!wait1(&B.acc_empty[a], aph ^ 1, B, P.status)) { ok = false; break; }
         ptx::tc_fence_after();
         const uint32_t d = tmem + (uint32_t)(a * BN2);
-        const int nch = min((J + 1) * BN2, ns_pad) / (BK * C::SUB);
+        const int nch = g2p_stages(ns, J);
         for (int ic = 0; ic < nch; ++ic) {
           if (!wait1(&B.full[s], ph, B, P.status) || !wait1(&B.ready[s], ph, B, P.status)) {
             ok = false;
             break;
           }
           ptx::tc_fence_after();
+          const int n = g2p_stage_cols(ns, J, ic);
+          const uint32_t dn = d + (uint32_t)(g2p_cols(ns, J) - n);
+          const uint32_t idesc = C::IDESC + ((uint32_t)n << 14);        // N >> 3 at bit 17
 #pragma unroll
           for (int c = 0; c < C::SUB; ++c)
-            issue_g2p_mmas<PREC>(d, ptx::smem_u32(smem + s * SB + c * C::CHUNK), ic == 0 && c == 0);
+            issue_g2p_mmas<PREC>(dn, ptx::smem_u32(smem + s * SB + c * C::CHUNK), idesc, ic == 0 && c == 0);
           ptx::mma_commit_pair_mc(&B.empty[s], PAIR_MASK);
           if (++s == STAGES) { s = 0; ph ^= 1; }
         }
@@ -660,10 +747,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     for (int item = pair; item < items && ok; item += npairs) {
       int q, k, R2, jp, j0, j1;
       const TcProblem* pr = g2_item<BN2>(P, item, q, k, R2, jp, j0, j1);
-      const int ns_pad = pr->ns_pad;
+      const int ns = g2p_ns(pr);
       for (int jj = j0; jj < j1 && ok; ++jj) {
         const int J = g2_tile(P, q, jj);
-        const int nch = min((J + 1) * BN2, ns_pad) / (BK * C::SUB);
+        const int nch = g2p_stages(ns, J);
         for (int ic = 0; ic < nch; ++ic) {
           if (!wait1(&B.full[s], ph, B, P.status)) { ok = false; break; }
           ptx::mbar_arrive_cluster(&B.ready[s], 0);
@@ -671,26 +758,70 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
       }
     }
-  } else if (warp >= 2) {
-    // ---------------- row-dot epilogue (both CTAs; TMEM lane quarter = warp % 4) ----------------
-    const int lq = warp & 3;
-    const int row = lq * 32 + lane;
-    int a = 0;
-    uint32_t aph = 0;
+  } else if (warp == 6 && lane == 0) {
+    // ---------------- TMA of the row-dot's Psi chunks (both CTAs) ----------------
+    for (int q = 0; q < P.nslot; ++q) {
+      const TcProblem* pr = P.probs + P.pid[q];
+      ptx::tmap_acquire(&pr->g2a0);
+      if (PARTS == 2) ptx::tmap_acquire(&pr->g2a1);
+    }
+    int s = 0;
+    uint32_t ph = 0;
+    int pending[C::ESTAGES];
+    for (int i = 0; i < C::ESTAGES; ++i) pending[i] = -1;
     bool ok = true;
     for (int item = pair; item < items && ok; item += npairs) {
       int q, k, R2, jp, j0, j1;
       const TcProblem* pr = g2_item<BN2>(P, item, q, k, R2, jp, j0, j1);
-      const int ns_pad = pr->ns_pad;
-      const long long Ng = pr->Ng;
+      const int ns = g2p_ns(pr);
+      const int rb = 2 * R2 + rank;
+      for (int jj = j0; jj < j1 && ok; ++jj) {
+        const int J = g2_tile(P, q, jj);
+        const int n = g2p_cols(ns, J) / 32;
+        for (int c = 0; c < n; ++c) {
+          if (!wait1(&eempty[s], ph ^ 1, B, P.status)) { ok = false; break; }
+          uint8_t* st = smem + C::E_OFF + s * C::ESB;
+          const int i0 = J * BN2 + c * 32;
+          ptx::mbar_arrive_expect_tx(&efull[s], C::ESB);
+          ptx::tma_load_2d(st, &pr->g2a0, &efull[s], i0, rb * BM);
+          if (PARTS == 2) ptx::tma_load_2d(st + TILE_A, &pr->g2a1, &efull[s], i0, rb * BM);
+          else ptx::tma_load_2d(st + TILE_A, &pr->g2a0, &efull[s], i0 + BK, rb * BM);
+          pending[s] = (int)ph;
+          if (++s == C::ESTAGES) { s = 0; ph ^= 1; }
+        }
+      }
+    }
+    for (int i = 0; i < C::ESTAGES; ++i)
+      if (pending[i] >= 0) wait_drain(&efull[i], (uint32_t)pending[i]);
+  } else if (warp >= 2 && warp < 6) {
+    // ---------------- row-dot epilogue (both CTAs; TMEM lane quarter = warp % 4) ----------------
+    const int lq = warp & 3;
+    const int row = lq * 32 + lane;
+    int a = 0, es = 0;
+    uint32_t aph = 0, eph = 0;
+    bool ok = true;
+    for (int item = pair; item < items && ok; item += npairs) {
+      int q, k, R2, jp, j0, j1;
+      const TcProblem* pr = g2_item<BN2>(P, item, q, k, R2, jp, j0, j1);
+      const int ns = g2p_ns(pr);
       const long long r = (long long)(2 * R2 + rank) * BM + row;
       double acc_row = 0.0;
-      for (int jj = j0; jj < j1; ++jj) {
+      for (int jj = j0; jj < j1 && ok; ++jj) {
         const int J = g2_tile(P, q, jj);
         if (!waitw(&B.acc_full[a], aph, B, P.status)) { ok = false; break; }
         ptx::tc_fence_after();
         const uint32_t tb = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(a * BN2);
-        const float part = g2_tile_dot<PREC, BN2>(tb, J, r, Ng, ns_pad, pr->psi0, pr->psi1);
+        const int n = g2p_cols(ns, J) / 32;
+        float part = 0.f;
+        for (int c = 0; c < n; ++c) {
+          float v[32];
+          ptx::tmem_ld32(tb + c * 32, v);
+          if (!waitw(&efull[es], eph, B, P.status)) { ok = false; break; }
+          part = g2p_dot<PREC>(part, v, ptx::smem_u32(smem + C::E_OFF + es * C::ESB), row);
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(&eempty[es]);
+          if (++es == C::ESTAGES) { es = 0; eph ^= 1; }
+        }
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive_cluster(&B.acc_empty[a], 0);
@@ -1595,10 +1726,12 @@ bool build_problem(const Channel& c, const SysState& S, int ch, TcProblem& pr) {
   const uint64_t dB2[3] = {(uint64_t)c.ns_pad, (uint64_t)c.ns_pad, (uint64_t)S.kmax};
   const uint64_t sB2[2] = {(uint64_t)c.ns_pad * eb, (uint64_t)c.ns_pad * c.ns_pad * eb};
   const uint32_t bB2[3] = {(uint32_t)BK, 128, 1};            // GEMM2 B: 128-row boxes
+  const uint32_t bC2[3] = {(uint32_t)BK, 64, 1};             // and 64-row boxes (narrow stages)
   if (!make_map(&pr.g1a, ta, 4, 4, d1, sa, bA1, swa) || !make_map(&pr.g1b0, t0, eb, 4, d1, s1, bA1) ||
       !make_map(&pr.g1b1, t1, eb, 4, d1, s1, bA1) ||
       !make_map(&pr.g2a0, r0, eb, 2, dA2, sA2, bA2) || !make_map(&pr.g2a1, r1, eb, 2, dA2, sA2, bA2) ||
-      !make_map(&pr.g2b0, x0, eb, 3, dB2, sB2, bB2) || !make_map(&pr.g2b1, x1, eb, 3, dB2, sB2, bB2))
+      !make_map(&pr.g2b0, x0, eb, 3, dB2, sB2, bB2) || !make_map(&pr.g2b1, x1, eb, 3, dB2, sB2, bB2) ||
+      !make_map(&pr.g2c0, x0, eb, 3, dB2, sB2, bC2) || !make_map(&pr.g2c1, x1, eb, 3, dB2, sB2, bC2))
     return false;
   pr.Ng = S.Ng;
   pr.a_stride = (long long)S.nspin * S.Ng_pad;
@@ -1743,7 +1876,7 @@ int pair_clusters() {
 
 template <int PREC>
 int pair_clusters_g2() {
-  return cluster_pairs(k_gemm2_pair<PREC>, G2PCfg<PREC>::SMEM, NTHREADS, PairKernels<PREC>::g2_attr,
+  return cluster_pairs(k_gemm2_pair<PREC>, G2PCfg<PREC>::SMEM, G2PCfg<PREC>::THREADS, PairKernels<PREC>::g2_attr,
                        PairKernels<PREC>::g2_cache, "response");
 }
 
@@ -1976,7 +2109,12 @@ cudaError_t gemm2_pair_group(const TcEntry* e, int n, int out_io, int out_is_io,
     P.nslot = q;
     P.begin[q] = items;
     if (items == 0) continue;
-    P.sync = sync && q == 1 && P.nsplit[0] == 1 ? sync : nullptr;
+    // round alignment: one problem, unsplit items, and only where the operands
+    // of a round outgrow L2 (at 96^3 / 4096: 384 ms with, 461 without); over
+    // short items the grid-wide wait at each round costs more than the shared
+    // rows save (48^3 / 512, K = 8: 515 us without, 582 with; 64^3 / 1024:
+    // 8.0 ms and 8.7; equal at 72^3 / 2048)
+    P.sync = sync && q == 1 && P.nsplit[0] == 1 && hp[0]->ns_pad >= 2048 ? sync : nullptr;
     if (P.sync && (err = cudaMemsetAsync(P.sync, 0, sizeof(unsigned), st)) != cudaSuccess) return err;
     const int clusters = pair_clusters_g2<PREC>();
     const int pairs = items < clusters ? items : clusters;
@@ -1987,7 +2125,7 @@ cudaError_t gemm2_pair_group(const TcEntry* e, int n, int out_io, int out_is_io,
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(2 * pairs, 1, 1);
-    cfg.blockDim = dim3(NTHREADS, 1, 1);
+    cfg.blockDim = dim3(C::THREADS, 1, 1);
     cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;
     cfg.attrs = at;

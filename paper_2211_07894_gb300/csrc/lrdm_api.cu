@@ -547,6 +547,11 @@ lrdm_status autotune(lrdm_ctx* ctx, cudaStream_t st) {
   cudaError_t err = cudaSuccess;
   TcTune best = ctx->tune;
   float tbest = 1e30f;
+  // The pair forms are candidates where a launch gives every CTA pair an item.
+  // Below that one item per pair or per SM is all there is and the forms time
+  // within two microseconds of one another (12 x 11 x 10, 3 points x 300 columns, K = 4:
+  // 72 response items for 76 pairs: 18.7 us on pairs, 20.5 on single CTAs).
+  const long long units = tc_pair_units(ctx->opt.prec);
   const int g1_cand[4][2] = {{G1_PAIR, 1}, {256, 1}, {128, 1}, {128, 2}};   // (MMA width, directions per tile)
   const TcTune start = ctx->tune;
   for (const auto& c : g1_cand) {
@@ -560,6 +565,11 @@ lrdm_status autotune(lrdm_ctx* ctx, cudaStream_t st) {
     for (size_t e = 0; e < g1.size(); ++e)
       if (g1_sys[e] >= 0) g1[e].split = choose_split(ctx, g1_sys[e], g1[e].K);
     ctx->tune = start;
+    if (c[0] == G1_PAIR) {
+      long long items = 0;
+      for (const TcEntry& x : g1) items += (long long)x.host->ntiles_p * x.K * (x.split > 1 ? x.split : 1);
+      if (items < units) continue;
+    }
     const float ms = time_launch([&] { return launch_gemm1_tc_group(ctx->opt.prec, g1.data(), (int)g1.size(),
                                                                     ctx->d_status, st, t, G1_NCH_CAP, 0,
                                                                     ctx->d_round); },
@@ -568,7 +578,9 @@ lrdm_status autotune(lrdm_ctx* ctx, cudaStream_t st) {
     if (ms < tbest) { tbest = ms; best.g1_nb = c[0]; best.g1_dpt = c[1]; }
   }
   tbest = 1e30f;
-  for (int bn = 128; bn <= G2_PAIR; bn *= 2)          // 128, 256, and 256 on CTA pairs
+  long long g2_items = 0;
+  for (const TcEntry& x : g2) g2_items += (long long)((x.host->nR + 1) / 2) * x.K;
+  for (int bn = 128; bn <= (g2_items < units ? 256 : G2_PAIR); bn *= 2)   // 128, 256, and 256 on CTA pairs
     for (int kg = 1; kg <= 4; kg *= 2) {
       TcTune t = ctx->tune;
       t.g2_bn = bn;

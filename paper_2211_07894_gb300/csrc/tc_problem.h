@@ -11,7 +11,8 @@ namespace lrdm {
 struct TcProblem {
   CUtensorMap g1a;                      // GEMM1 A: Psi^T tile-major FP32 (TF32: rounded), box 128 rows
   CUtensorMap g1b0, g1b1;               // GEMM1 B: Psi^T tile-major bf16 hi / lo (TF32: = A)
-  CUtensorMap g2a0, g2a1, g2b0, g2b1;   // GEMM2: Psi rows (A), X'' [k_max][j][i] (B)
+  CUtensorMap g2a0, g2a1, g2b0, g2b1;   // GEMM2: Psi rows (A), X'' [k_max][j][i] (B), boxes of 128 rows
+  CUtensorMap g2c0, g2c1;               // GEMM2: X'' in boxes of 64 rows
   long long Ng;                          // grid points
   long long a_stride;                    // direction stride of the GEMM1 weights
   const float* a;                        // GEMM1 weights of this channel (direction 0)
