@@ -433,8 +433,8 @@ void lrdm_lrdma_destroy(lrdm_lrdma* a);
  *   X_kappa = Psi_kappa^H diag(w dV_k) Psi_kappa,
  *   sum_kappa w_kappa sum_i L_kappa,ii (X_kappa,ii - mu') = 0,
  *   drho_k = g sum_kappa w_kappa diag(Psi_kappa L_kappa o (X_kappa - mu' I) Psi_kappa^H).
- * Spin-restricted.  FP64 / FP32 run complex contractions on the CUDA cores;
- * TF32 / BF16X3 run the real tensor-core contractions on the stacked operand
+ * Spin-restricted.  Every precision runs the real contractions (CUDA cores in
+ * FP64 / FP32, tensor cores in TF32 / BF16X3) on the stacked operand
  * C = [Re Psi, Im Psi] (N_g x 2 N_s): C^T diag(a) C holds Re X and Im X, and
  * the density is diag(C M C^T) with M = [[Re G, Im G], [-Im G, Re G]],
  * G = L o (X - mu' I).  A k-point context serves lrdm_kp_gateaux,
@@ -482,8 +482,8 @@ lrdm_status lrdm_kp_create(lrdm_ctx** out, const lrdm_kpoint_system* sys, const 
 lrdm_status lrdm_kp_gateaux(lrdm_ctx* ctx, const void* v, int K, void* f_out, double* dmu_out,
                             void* stream);
 /* The number of grid-row ranges the projection of a K-direction call is
- * split into (tensor cores: chosen per call to fill the persistent grid's
- * waves, at most 4; CUDA cores: fixed at create).  For measurement. */
+ * split into, chosen per call (tensor cores: to fill the persistent grid's
+ * waves, at most 4; CUDA cores: to fill the SMs).  For measurement. */
 lrdm_status lrdm_kp_get_split(lrdm_ctx* ctx, int K, int* split);
 
 /* Copies the projected perturbation X_k = Psi^T diag(w dV_k) Psi of direction

@@ -13,11 +13,6 @@ namespace {
 __device__ __forceinline__ double ld_c(const void* p, int fp64, long long i) {
   return fp64 ? static_cast<const double*>(p)[i] : (double)static_cast<const float*>(p)[i];
 }
-__device__ __forceinline__ void st_c(void* p, int fp64, long long i, double x) {
-  if (fp64) static_cast<double*>(p)[i] = x;
-  else static_cast<float*>(p)[i] = (float)x;
-}
-
 inline int grid_for(long long n, int block) {
   long long b = (n + block - 1) / block;
   if (b > 152LL * 32) b = 152LL * 32;
@@ -271,9 +266,9 @@ __global__ void k_dmu(DmuArgs A, int acc64, double* __restrict__ dmu, double* __
   for (int s = 0; s < A.nspin; ++s) {
     long long mat = (long long)A.ldx[s] * A.ldx[s];
     for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
-      double x = 0.0;
-      for (int p = 0; p < A.nsplit; ++p)
-        x += ld_c(A.X[s], acc64, ((long long)p * A.K + k) * mat + (long long)i * A.ldx[s] + i);
+      const long long o = k * mat + (long long)i * A.ldx[s] + i;
+      const double x = acc64 ? sum_strided(static_cast<const double*>(A.X[s]) + o, A.nsplit, A.K * mat)
+                             : sum_strided(static_cast<const float*>(A.X[s]) + o, A.nsplit, A.K * mat);
       double l = A.L[s][(long long)i * A.ns[s] + i];
       num += l * x;
       den += l;
@@ -297,51 +292,24 @@ __global__ void k_dmu(DmuArgs A, int acc64, double* __restrict__ dmu, double* __
   }
 }
 
-// X'' in one of three layouts:
-//   layout 0: out[k][i][j] (ld = ns)        -- CUDA-core GEMM2, compute type
-//   layout 1: out[k][j][i] (ld = ns_pad) fp32 -- TF32 GEMM2 B operand (K-major)
-//   layout 2: out_hi/out_lo[k][j][i] bf16     -- BF16X3 GEMM2 B operand (K-major)
-// value c_ij * (L_ij (X_ij - delta_ij shift_k)) with c = 2, 1, 0 for i <, =, > j.
-// Adjoint form (adjoint = 1): L_ij G_ij - delta_ij L_ii shift_k * inv_trace.
-// X is the full symmetric matrix (GEMM1 writes both triangles), summed over splits.
-__global__ void k_loewner_scale(const void* __restrict__ X, int acc64, int nsplit, int K, int ns,
-                                int ldx, const double* __restrict__ L,
-                                const double* __restrict__ shift, int adjoint, double inv_trace,
-                                int layout, int ldo, void* __restrict__ out,
-                                __nv_bfloat16* __restrict__ out_lo) {
-  long long mat_x = (long long)ldx * ldx;
-  long long mat_o = (long long)ldo * ldo;
-  GRID_STRIDE(e, (long long)K * mat_o) {
-    long long k = e / mat_o, rem = e - k * mat_o;
-    int row = (int)(rem / ldo), col = (int)(rem - (long long)row * ldo);
-    // layout 0: (row, col) = (i, j);  layouts 1, 2: (row, col) = (j, i)
-    int i = layout == 0 ? row : col;
-    int j = layout == 0 ? col : row;
-    double val = 0.0;
-    if (i < ns && j < ns && i <= j) {
-      double x = 0.0;
-      // read the (row, col) entry: X and L are symmetric
-      for (int p = 0; p < nsplit; ++p)
-        x += ld_c(X, acc64, ((long long)p * K + k) * mat_x + (long long)row * ldx + col);
-      double l = L[(long long)row * ns + col];
-      double xp;
-      if (adjoint) xp = l * x - (i == j ? l * shift[k] * inv_trace : 0.0);
-      else xp = l * (x - (i == j ? shift[k] : 0.0));
-      val = (i == j ? 1.0 : 2.0) * xp;
-    }
-    if (layout == 0) {
-      st_c(out, acc64, e, val);
-    } else if (layout == 1) {
-      uint32_t t;
-      asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"((float)val));
-      static_cast<float*>(out)[e] = __uint_as_float(t);
-    } else {
-      float v32 = (float)val;
-      __nv_bfloat16 hi = __float2bfloat16_rn(v32);
-      static_cast<__nv_bfloat16*>(out)[e] = hi;
-      out_lo[e] = __float2bfloat16_rn(v32 - __bfloat162float(hi));
-    }
-  }
+// X'' of the CUDA-core GEMM2: out[k][i][j] = c_ij (L_ij (X_ij - delta_ij shift_k)),
+// c = 2 for i < j, 1 on the diagonal; below it the buffer keeps the zeros it was
+// created with.  Adjoint form (adjoint = 1): L_ij G_ij - delta_ij L_ii shift_k *
+// inv_trace.  X summed over the row ranges; products in FP64.
+template <typename Tc>
+__global__ void k_loewner_scale(const Tc* __restrict__ X, int nsplit, int K, int ns,
+                                const double* __restrict__ L, const double* __restrict__ shift,
+                                int adjoint, double inv_trace, Tc* __restrict__ out) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = blockIdx.y, k = blockIdx.z;
+  if (j >= ns || j < i) return;
+  const long long mat = (long long)ns * ns, o = (long long)k * mat + (long long)i * ns + j;
+  const double x = sum_strided(X + o, nsplit, (long long)K * mat);
+  const double l = L[(long long)i * ns + j];
+  double xp;
+  if (adjoint) xp = l * x - (i == j ? l * shift[k] * inv_trace : 0.0);
+  else xp = l * (x - (i == j ? shift[k] : 0.0));
+  out[o] = (Tc)(i == j ? xp : 2.0 * xp);
 }
 
 // X'' for the tensor-core response GEMM: entry (k, row = j, col = i) =
@@ -425,9 +393,9 @@ __global__ void k_trace_bar(DmuArgs A, int acc64, double* __restrict__ tbar) {
   for (int s = 0; s < A.nspin; ++s) {
     long long mat = (long long)A.ldx[s] * A.ldx[s];
     for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
-      double x = 0.0;
-      for (int p = 0; p < A.nsplit; ++p)
-        x += ld_c(A.X[s], acc64, ((long long)p * A.K + k) * mat + (long long)i * A.ldx[s] + i);
+      const long long o = k * mat + (long long)i * A.ldx[s] + i;
+      const double x = acc64 ? sum_strided(static_cast<const double*>(A.X[s]) + o, A.nsplit, A.K * mat)
+                             : sum_strided(static_cast<const float*>(A.X[s]) + o, A.nsplit, A.K * mat);
       num += A.L[s][(long long)i * A.ns[s] + i] * x;
     }
   }
@@ -738,14 +706,14 @@ static DmuArgs dmu_args(const SysState& S, const void* const* X, int K) {
 cudaError_t launch_dmu(const SysState& S, const void* const* Xparts, int K, int acc_fp64,
                        double* dmu, double* dmu_out, int* status, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  k_dmu<<<K, 256, 0, st>>>(dmu_args(S, Xparts, K), acc_fp64, dmu, dmu_out, status);
+  k_dmu<<<K, 1024, 0, st>>>(dmu_args(S, Xparts, K), acc_fp64, dmu, dmu_out, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_trace_bar(const SysState& S, const void* const* Gparts, int K, int acc_fp64,
                              double* tbar, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  k_trace_bar<<<K, 256, 0, st>>>(dmu_args(S, Gparts, K), acc_fp64, tbar);
+  k_trace_bar<<<K, 1024, 0, st>>>(dmu_args(S, Gparts, K), acc_fp64, tbar);
   return cudaGetLastError();
 }
 
@@ -764,12 +732,13 @@ cudaError_t launch_loewner_scale(const SysState& S, int s, const void* Xpart, in
                                               static_cast<__nv_bfloat16*>(c.Xpp_lo));
     return cudaGetLastError();
   }
-  int ldx = c.ns;
-  int ldo = c.ns;
-  long long tot = (long long)K * ldo * ldo;
-  k_loewner_scale<<<grid_for(tot, 256), 256, 0, st>>>(
-      Xpart, acc_fp64, S.nsplit, K, c.ns, ldx, c.L, shift, adjoint, inv_trace_L, layout, ldo,
-      c.Xpp, static_cast<__nv_bfloat16*>(c.Xpp_lo));
+  const dim3 grid((unsigned)((c.ns + 127) / 128), (unsigned)c.ns, (unsigned)K);
+  if (acc_fp64)
+    k_loewner_scale<double><<<grid, 128, 0, st>>>(static_cast<const double*>(Xpart), S.nsplit, K, c.ns, c.L,
+                                                  shift, adjoint, inv_trace_L, static_cast<double*>(c.Xpp));
+  else
+    k_loewner_scale<float><<<grid, 128, 0, st>>>(static_cast<const float*>(Xpart), S.nsplit, K, c.ns, c.L,
+                                                 shift, adjoint, inv_trace_L, static_cast<float*>(c.Xpp));
   return cudaGetLastError();
 }
 

@@ -84,21 +84,6 @@ __global__ void __launch_bounds__(256) k_gram(const T* __restrict__ F, const T* 
 // (all with the elimination; 2e-15 with the Jacobi rotations).
 constexpr long long LS_N32 = 65536;
 
-// A value as an unevaluated sum s + c of two FP32 words.
-struct Pair32 {
-  float s, c;
-};
-// s + r = a + b exactly (Knuth)
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& r) {
-  s = __fadd_rn(a, b);
-  const float z = __fsub_rn(s, a);
-  r = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
-}
-__device__ __forceinline__ void pair_add(Pair32& a, const Pair32& b) {
-  float r;
-  two_sum(a.s, b.s, a.s, r);
-  a.c = __fadd_rn(a.c, __fadd_rn(b.c, r));
-}
 __device__ __forceinline__ Pair32 warp_sum(Pair32 a) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {

@@ -232,38 +232,28 @@ lrdm_status setup_system(lrdm_ctx* ctx, int idx, const lrdm_system& in, cudaStre
     LRDM_CU(launch_convert_psi(in.psi[c], o.io_dtype, in.ld_psi[c], S.Ng, ns, ch, prec, S.Ng_pad, st));
   }
 
-  // split of the grid reduction for the CUDA-core GEMM1 (enough blocks to fill
-  // 152 SMs twice); the tensor-core GEMM1 reduces the whole grid per tile.
-  if (!is_tc(prec)) {
-    int nt = (S.ch[0].ns + SIMT_TILE - 1) / SIMT_TILE;
-    long long blocks = (long long)nt * (nt + 1) / 2 * S.kmax;
-    long long want = (2LL * 152 * 2 + blocks - 1) / blocks;
-    long long maxsplit = S.Ng / 256 > 0 ? S.Ng / 256 : 1;
-    if (want > maxsplit) want = maxsplit;
-    if (want > 64) want = 64;
-    // row-sharded: one partial X per rank, summed over the ranks as it is
-    S.nsplit = ctx->rows ? 1 : (int)(want < 1 ? 1 : want);
-  } else {
-    S.nsplit = 1;
-  }
+  S.nsplit = 1;                    // chosen per call
 
   // workspaces
   const int accsz = fp64 ? 8 : 4;
-  // tensor cores: the X / G buffers hold up to 8 grid-row partials of a
-  // k_max-direction call while they stay within 512 MB per channel, so that
-  // small subspaces (few tiles) can split their grid reduction at any K
+  // the X / G buffers hold several grid-row partials of a k_max-direction call
+  // while they stay within 512 MB per channel, so that few tiles (a small
+  // subspace) can split their grid reduction: up to 8 on the tensor cores, on
+  // the CUDA cores the count simt_split takes (row-sharded: one per rank)
   S.xslots = S.kmax;
-  if (is_tc(prec)) {
+  {
     size_t ldmax = 0;
-    for (int c = 0; c < in.nspin; ++c) ldmax = std::max(ldmax, (size_t)S.ch[c].ns_pad);
+    for (int c = 0; c < in.nspin; ++c)
+      ldmax = std::max(ldmax, (size_t)(is_tc(prec) ? S.ch[c].ns_pad : S.ch[c].ns));
     const size_t per = (size_t)S.kmax * ldmax * ldmax * accsz;
-    const size_t cap = std::min<size_t>(8, std::max<size_t>(1, (512ull << 20) / per));
-    S.xslots = (int)(cap * S.kmax);
+    const int room = (int)std::min<size_t>(64, std::max<size_t>(1, (512ull << 20) / per));
+    if (is_tc(prec)) S.xslots = std::min(8, room) * S.kmax;
+    else if (!ctx->rows) S.xslots = simt_split(fp64, S.ch[0].ns, S.Ng, S.kmax, room * S.kmax) * S.kmax;
   }
   for (int c = 0; c < in.nspin; ++c) {
     Channel& ch = S.ch[c];
     const size_t ldx = is_tc(prec) ? ch.ns_pad : ch.ns;
-    const size_t xcount = (size_t)S.nsplit * (is_tc(prec) ? S.xslots : S.kmax) * ldx * ldx;
+    const size_t xcount = (size_t)S.xslots * ldx * ldx;
     LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ch.Xpart), xcount * accsz));
     LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ch.Gpart), xcount * accsz));
     const size_t pcount = (size_t)S.kmax * ldx * ldx;
@@ -341,8 +331,15 @@ lrdm_status gemm2_simt(lrdm_ctx* ctx, SysState& S, int c, int K, double factor, 
   count(ctx, 1);
   const void* psi = prec == LRDM_FP64 ? static_cast<const void*>(ch.psi64)
                                       : static_cast<const void*>(ch.psi32);
-  cudaError_t e = launch_gemm2_simt(prec == LRDM_FP64, psi, ch.ns, S.Ng, ch.Xpp, K, factor, v,
-                                    v_stride, out, out_stride, ctx->opt.io_dtype, out_is_io, st);
+  SimtOut o;
+  o.mode = out_is_io ? SIMT_OUT_F : SIMT_OUT_C;
+  o.f64 = out_is_io ? ctx->opt.io_dtype == LRDM_DTYPE_F64 : prec == LRDM_FP64;
+  o.factor = factor;
+  o.out = out;
+  o.stride = out_stride;
+  o.v = v;
+  o.v_stride = v_stride;
+  cudaError_t e = launch_gemm2_simt(prec == LRDM_FP64, psi, ch.ns, S.Ng, ch.Xpp, K, o, st);
   prof_end(ctx, pi, st);
   return from_cuda(e);
 }
@@ -382,7 +379,9 @@ lrdm_status tc_group(lrdm_ctx* ctx, int gemm, int out_is_io, cudaStream_t st) {
 // (1360 items, 0.994 of 9 waves, against 0.895 for 1-4 ranges).
 int choose_split(lrdm_ctx* ctx, int s, int K) {
   const SysState& S = ctx->sys[s];
-  if (!is_tc(ctx->opt.prec) || K <= 0 || ctx->tc_pid.empty() || ctx->rows) return 1;
+  if (K <= 0 || ctx->rows) return 1;
+  if (!is_tc(ctx->opt.prec)) return simt_split(ctx->opt.prec == LRDM_FP64, S.ch[0].ns, S.Ng, K, S.xslots);
+  if (ctx->tc_pid.empty()) return 1;
   const TcProblem& pr = ctx->tc_host[ctx->tc_pid[2 * s]];
   const bool pair = ctx->tune.g1_nb == G1_PAIR;
   const bool wide = ctx->tune.g1_nb == 256;
@@ -671,9 +670,11 @@ lrdm_status forward_all(lrdm_ctx* ctx, const void* const* v, const int* K, void*
     }
     LRDM_CK(tc_group(ctx, 1, 0, st));
   } else {
-    for (int s = 0; s < ctx->nsys; ++s)
+    for (int s = 0; s < ctx->nsys; ++s) {
+      if (K[s] > 0) ctx->sys[s].nsplit = choose_split(ctx, s, K[s]);
       for (int c = 0; c < ctx->sys[s].nspin && K[s] > 0; ++c)
         LRDM_CK(gemm1_simt(ctx, ctx->sys[s], c, K[s], ctx->sys[s].ch[c].Xpart, st));
+    }
   }
   LRDM_CK(reduce_projections(ctx, K, false, st));
   // mu' and the Loewner scaling

@@ -24,22 +24,35 @@ __device__ __forceinline__ float tf32_rna(float x) {
   return __uint_as_float(t);
 }
 
-// Four consecutive shared-memory values (16-byte aligned) with 128-bit loads:
-// the register tiles of the CUDA-core contractions.
-__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
-  const float4 t = *reinterpret_cast<const float4*>(p);
-  v[0] = t.x;
-  v[1] = t.y;
-  v[2] = t.z;
-  v[3] = t.w;
+// A value as an unevaluated sum s + c of two FP32 words.
+struct Pair32 {
+  float s, c;
+};
+// s + r = a + b exactly (Knuth)
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& r) {
+  s = __fadd_rn(a, b);
+  const float z = __fsub_rn(s, a);
+  r = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
 }
-__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
-  const double2 a = *reinterpret_cast<const double2*>(p);
-  const double2 b = *reinterpret_cast<const double2*>(p + 2);
-  v[0] = a.x;
-  v[1] = a.y;
-  v[2] = b.x;
-  v[3] = b.y;
+__device__ __forceinline__ void pair_add(Pair32& a, const Pair32& b) {
+  float r;
+  two_sum(a.s, b.s, a.s, r);
+  a.c = __fadd_rn(a.c, __fadd_rn(b.c, r));
+}
+// Sum of n values p[0], p[stride], ..: FP64 data in FP64, FP32 data as an FP32
+// pair (48 bits; one FP64 addition and one conversion a value cost 128 FP32
+// operations on GB300).
+__device__ __forceinline__ double sum_strided(const double* __restrict__ p, int n, long long stride) {
+  double x = 0.0;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i) x += p[i * stride];
+  return x;
+}
+__device__ __forceinline__ double sum_strided(const float* __restrict__ p, int n, long long stride) {
+  Pair32 x{p[0], 0.f};
+#pragma unroll 4
+  for (int i = 1; i < n; ++i) pair_add(x, Pair32{p[i * stride], 0.f});
+  return (double)x.s + (double)x.c;
 }
 
 // NVTX range for the profilers' timelines (one per API call and per phase of
@@ -59,7 +72,6 @@ enum : int {
 };
 
 constexpr int KMAX_LIMIT = 64;       // directions per system per call
-constexpr int SIMT_TILE = 64;        // CUDA-core GEMM tile edge (states)
 constexpr int LS_CHUNK = 64;         // grid points per staged chunk in the Gram kernel
 constexpr int LS_BLOCKS = 304;       // 2 x 152 SMs
 constexpr int UPD_BLOCKS = 608;
@@ -106,10 +118,9 @@ struct SysState {
   double w = 0, g = 2, kT = 0, ne = 0, mu = 0;
   bool occ_given = false;
   Channel ch[2];
-  int xslots = 0;                    // tensor cores: direction slots of the X / G buffers (>= kmax;
-                                     // grid-row partials of a K-direction call use nsplit * K of them)
-  int nsplit = 1;                    // grid-row splits of GEMM1 (CUDA cores: fixed at create;
-                                     // tensor cores: chosen per call from K, nsplit * K <= xslots)
+  int xslots = 0;                    // direction slots of the X / G buffers (>= kmax; grid-row
+                                     // partials of a K-direction call use nsplit * K of them)
+  int nsplit = 1;                    // grid-row splits of GEMM1, chosen per call from K
   // Poisson
   cufftHandle plan_r2c = 0, plan_c2r = 0;
   bool plans = false;
@@ -170,12 +181,12 @@ struct lrdm_ctx {
   // Brillouin-zone-sampled system (lrdm_kp_create): one periodic system, nk
   // complex subspaces sharing mu, the grid and the Poisson plans of sys[0]
   bool kp = false;
-  int kp_nk = 0, kp_ns = 0, kp_nsplit = 1;
+  int kp_nk = 0, kp_ns = 0;
   std::vector<double> kp_w;          // BZ weights
-  std::vector<void*> kp_pr, kp_pi;   // [nk] Psi planes [N_g][N_s] compute type
+  std::vector<void*> kp_C;           // CUDA cores: [nk] stacked C = [Re Psi, Im Psi], [N_g][2 N_s]
   std::vector<double*> kp_eps, kp_occ, kp_L;
-  std::vector<void*> kp_Xr, kp_Xi;   // [nk] [nsplit][kmax][N_s][N_s]
-  std::vector<void*> kp_Yr, kp_Yi;   // [nk] [kmax][N_s][N_s] Loewner-scaled
+  std::vector<void*> kp_P;           // [nk] [xslots][2 N_s][2 N_s]: C^T diag(a) C
+  std::vector<void*> kp_Y;           // [nk] [kmax][2 N_s][2 N_s] Loewner-scaled
   double* kp_drho = nullptr;         // [kmax][N_g] FP64 accumulator
   // tensor-core modes: per k-point the stacked real operand C = [Re Psi, Im Psi]
   // (N_g x 2 N_s) as one channel of the real contractions, its problem index
@@ -205,30 +216,22 @@ cudaError_t launch_loewner_f32(const double* L, int ns, int ns_pad, float* Lf, c
 // ---------------- Brillouin-zone-sampled response (k_kpoint.cu) ----------------
 constexpr int KP_MAX = 32;           // k-points per context
 struct KpDmuArgs {
-  const void* Xr[KP_MAX];            // Re X (CUDA cores) or the stacked Gram P (tensor cores)
+  const void* P[KP_MAX];             // the stacked Gram: Re X_ii = P_ii + P_(ns+i)(ns+i)
   const double* L[KP_MAX];
   double kw[KP_MAX];
   int nk, ns, K, nsplit, fp64;
-  int ld;                            // leading dimension of the X planes
-  int stacked;                       // 1: Re X_ii = P_ii + P_(ns+i)(ns+i)
+  int ld;                            // leading dimension of P
 };
 struct KpSumArgs {
   const float* part[KP_MAX];         // [K][N_g] per k-point, factor included
   int nk;
 };
-// X_kappa (re, im) = Psi^H diag(a_k) Psi over nsplit grid-row ranges
-cudaError_t launch_kp_gemm1(int fp64, const void* pr, const void* pi, int ns, long long Ng,
-                            const void* a, long long a_stride, int K, void* Xr, void* Xi, int nsplit,
-                            cudaStream_t st);
 // mu'_k from the BZ-averaged traceless condition
 cudaError_t launch_kp_dmu(const KpDmuArgs& A, double* dmu, double* dmu_out, cudaStream_t st);
-// Y = c L o conj(X - mu' I), upper part
-cudaError_t launch_kp_scale(int fp64, const void* Xr, const void* Xi, int nsplit, int K, int ns,
-                            const double* L, const double* dmu, void* Yr, void* Yi, cudaStream_t st);
-// drho[k] += factor * Re diag-form of Y over Psi
-cudaError_t launch_kp_gemm2(int fp64, const void* pr, const void* pi, int ns, long long Ng,
-                            const void* Yr, const void* Yi, int K, double factor, double* drho,
-                            cudaStream_t st);
+// CUDA-core modes: M'' [K][2 N_s][2 N_s] (upper part, compute type) from the
+// stacked Gram P [nsplit][K][2 N_s][2 N_s]
+cudaError_t launch_kp_scale(int fp64, const void* P, int nsplit, int K, int ns, const double* L,
+                            const double* dmu, void* Y, cudaStream_t st);
 cudaError_t launch_kp_finish(const double* drho, const void* v, int io, long long n, void* f,
                              cudaStream_t st);
 cudaError_t launch_kp_density(int fp64, const void* pr, const void* pi, int ns, int ld, long long Ng,
@@ -295,14 +298,28 @@ cudaError_t launch_eps_occ_bar(const SysState& S, int s, int K, int acc_fp64,
                                double* occ_bar, cudaStream_t st);
 
 // ---------------- CUDA-core GEMMs (k_simt.cu) ----------------
-// Xpart[split][q][i][j] (tiles I <= J) = sum_r psi[r][i] a[q][r] psi[r][j]
+// Xpart[split][q][i][j] = sum over the split's rows of psi[r][i] a[q][r] psi[r][j]
 cudaError_t launch_gemm1_simt(int fp64, const void* psi, int ns, long long Ng, const void* a,
                               long long a_stride, int nq, void* Xpart, int nsplit, cudaStream_t st);
-// out[q][r] = factor * sum_j sum_i psi[r][i] Xpp[q][i][j] psi[r][j] (- v[q][r] if sub_v)
+// Grid-row ranges of launch_gemm1_simt for K directions (at most slots / K)
+int simt_split(int fp64, int ns, long long Ng, int K, int slots);
+// Where GEMM2 puts factor * sum_j sum_{i <= j} psi[r][i] Xpp[q][i][j] psi[r][j]
+enum {
+  SIMT_OUT_F = 0,                    // out (io dtype) = value - v
+  SIMT_OUT_C = 1,                    // out (compute type) = value
+  SIMT_OUT_ADD = 2                   // out (FP64) += value
+};
+struct SimtOut {
+  int mode = SIMT_OUT_C;
+  int f64 = 0;                       // out (and v) are FP64 (modes F and C)
+  double factor = 1.0;
+  void* out = nullptr;
+  long long stride = 0;
+  const void* v = nullptr;
+  long long v_stride = 0;
+};
 cudaError_t launch_gemm2_simt(int fp64, const void* psi, int ns, long long Ng, const void* Xpp,
-                              int nq, double factor, const void* v, long long v_stride,
-                              void* out, long long out_stride, int out_io_dtype, int out_is_io,
-                              cudaStream_t st);
+                              int nq, const SimtOut& o, cudaStream_t st);
 
 // ---------------- least squares (k_ls.cu) ----------------
 // out = (t - sum_{k<K} <t, u_k> u_k) / ||.||_w (Krylov step, k_krylov.cu);

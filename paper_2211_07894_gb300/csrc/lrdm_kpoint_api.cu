@@ -90,6 +90,14 @@ int kp_choose_split(lrdm_ctx* ctx, int K) {
   return best;
 }
 
+// Grid-row ranges of the projection for K directions.
+int kp_split(lrdm_ctx* ctx, int K) {
+  const SysState& S = ctx->sys[0];
+  return is_tc(ctx->opt.prec)
+             ? kp_choose_split(ctx, K)
+             : simt_split(ctx->opt.prec == LRDM_FP64, 2 * ctx->kp_ns, S.Ng, K, S.xslots);
+}
+
 lrdm_status kp_response(lrdm_ctx* ctx, int K, double factor, double* dmu_out, cudaStream_t st) {
   NvtxRange nvtx_("k-point response");
   SysState& S = ctx->sys[0];
@@ -97,7 +105,7 @@ lrdm_status kp_response(lrdm_ctx* ctx, int K, double factor, double* dmu_out, cu
   const int fp64 = prec == LRDM_FP64;
   const bool tc = is_tc(prec);
   const int ns = ctx->kp_ns, nk = ctx->kp_nk;
-  const int split = tc ? kp_choose_split(ctx, K) : ctx->kp_nsplit;
+  const int split = kp_split(ctx, K);
   if (tc) {
     ctx->tc_entries.clear();
     for (int q = 0; q < nk; ++q) {
@@ -114,14 +122,13 @@ lrdm_status kp_response(lrdm_ctx* ctx, int K, double factor, double* dmu_out, cu
   } else {
     int pi = prof_begin(ctx, 1, st);
     for (int q = 0; q < nk; ++q)
-      LRDM_CU(launch_kp_gemm1(fp64, ctx->kp_pr[q], ctx->kp_pi[q], ns, S.Ng, S.a, S.Ng_pad, K, ctx->kp_Xr[q],
-                              ctx->kp_Xi[q], ctx->kp_nsplit, st));
+      LRDM_CU(launch_gemm1_simt(fp64, ctx->kp_C[q], 2 * ns, S.Ng, S.a, S.Ng_pad, K, ctx->kp_P[q], split, st));
     prof_end(ctx, pi, st);
     count(ctx, nk);
   }
   KpDmuArgs A{};
   for (int q = 0; q < nk; ++q) {
-    A.Xr[q] = tc ? ctx->kp_ch[q].Xpart : ctx->kp_Xr[q];
+    A.P[q] = tc ? ctx->kp_ch[q].Xpart : ctx->kp_P[q];
     A.L[q] = ctx->kp_L[q];
     A.kw[q] = ctx->kp_w[q];
   }
@@ -130,8 +137,7 @@ lrdm_status kp_response(lrdm_ctx* ctx, int K, double factor, double* dmu_out, cu
   A.K = K;
   A.nsplit = split;
   A.fp64 = fp64;
-  A.ld = tc ? ctx->kp_ch[0].ns_pad : ns;
-  A.stacked = tc ? 1 : 0;
+  A.ld = tc ? ctx->kp_ch[0].ns_pad : 2 * ns;
   LRDM_CU(launch_kp_dmu(A, S.dmu, dmu_out, st));
   count(ctx, 1);
   if (tc) {
@@ -156,12 +162,16 @@ lrdm_status kp_response(lrdm_ctx* ctx, int K, double factor, double* dmu_out, cu
   } else {
     LRDM_CU(cudaMemsetAsync(ctx->kp_drho, 0, (size_t)K * S.Ng * sizeof(double), st));
     for (int q = 0; q < nk; ++q)
-      LRDM_CU(launch_kp_scale(fp64, ctx->kp_Xr[q], ctx->kp_Xi[q], ctx->kp_nsplit, K, ns, ctx->kp_L[q], S.dmu,
-                              ctx->kp_Yr[q], ctx->kp_Yi[q], st));
+      LRDM_CU(launch_kp_scale(fp64, ctx->kp_P[q], split, K, ns, ctx->kp_L[q], S.dmu, ctx->kp_Y[q], st));
     int pi = prof_begin(ctx, 2, st);
-    for (int q = 0; q < nk; ++q)
-      LRDM_CU(launch_kp_gemm2(fp64, ctx->kp_pr[q], ctx->kp_pi[q], ns, S.Ng, ctx->kp_Yr[q], ctx->kp_Yi[q], K,
-                              factor * ctx->kp_w[q], ctx->kp_drho, st));
+    for (int q = 0; q < nk; ++q) {
+      SimtOut o;
+      o.mode = SIMT_OUT_ADD;
+      o.factor = factor * ctx->kp_w[q];
+      o.out = ctx->kp_drho;
+      o.stride = S.Ng;
+      LRDM_CU(launch_gemm2_simt(fp64, ctx->kp_C[q], 2 * ns, S.Ng, ctx->kp_Y[q], K, o, st));
+    }
     prof_end(ctx, pi, st);
     count(ctx, 2 * nk);
   }
@@ -263,28 +273,13 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
   for (int q = 0; q < nk; ++q)
     LRDM_CU(cudaMemcpy(eps[q].data(), in.eps[q], ns * sizeof(double), cudaMemcpyDeviceToHost));
   LRDM_CK(solve_mu_kp_host(eps, ctx->kp_w, S.ne, S.kT, S.g, &S.mu));
-  // CUDA cores: row ranges of the projection, about two blocks per SM at
-  // k_max directions; tensor cores: the whole grid per tile
-  ctx->kp_nsplit = 1;
-  if (!tc) {
-    const int nt = (ns + 63) / 64;
-    const long long blocks = (long long)nt * (nt + 1) / 2 * S.kmax;
-    const int sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
-    long long split = (2LL * sms + blocks - 1) / blocks;
-    if (split > S.Ng / 256) split = S.Ng / 256;
-    if (split > 64) split = 64;
-    ctx->kp_nsplit = (int)(split < 1 ? 1 : split);
-  }
   const size_t npsi = (size_t)S.Ng * ns, mat = (size_t)ns * ns;
-  ctx->kp_pr.assign(nk, nullptr);
-  ctx->kp_pi.assign(nk, nullptr);
+  ctx->kp_C.assign(nk, nullptr);
   ctx->kp_eps.assign(nk, nullptr);
   ctx->kp_occ.assign(nk, nullptr);
   ctx->kp_L.assign(nk, nullptr);
-  ctx->kp_Xr.assign(nk, nullptr);
-  ctx->kp_Xi.assign(nk, nullptr);
-  ctx->kp_Yr.assign(nk, nullptr);
-  ctx->kp_Yi.assign(nk, nullptr);
+  ctx->kp_P.assign(nk, nullptr);
+  ctx->kp_Y.assign(nk, nullptr);
   if (tc) {
     ctx->kp_ch.assign(nk, Channel());
     ctx->kp_pid.assign(nk, -1);
@@ -293,7 +288,12 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
   Channel& ch = S.ch[0];
   ch.ns = ns;
   LRDM_CK(dalloc(ctx, &ch.rho, S.Ng, false));
-  const size_t xc = (size_t)ctx->kp_nsplit * S.kmax * mat;
+  const size_t mat2 = 4 * mat;                 // the stacked Gram
+  if (!tc) {
+    // partial Grams within 512 MB per point
+    const int room = (int)std::min<size_t>(64, std::max<size_t>(1, (512ull << 20) / (S.kmax * mat2 * csz)));
+    S.xslots = simt_split(fp64, 2 * ns, S.Ng, S.kmax, room * S.kmax) * S.kmax;
+  }
   const int io = o.io_dtype;
   const size_t isz = io == LRDM_DTYPE_F64 ? sizeof(double) : sizeof(float);
   void* stack = nullptr;                       // tensor cores: [N_g][2 N_s] io dtype, set-up only
@@ -310,17 +310,15 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
       LRDM_CU(launch_loewner(ctx->kp_eps[q], ctx->kp_occ[q], ns, S.mu, S.kT, 0, o.degen_tol, 0,
                              ctx->kp_L[q], st));
       if (!tc) {
-        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_pr[q]), npsi * csz, false));
-        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_pi[q]), npsi * csz, false));
-        LRDM_CU(launch_kp_copy(fp64, in.psi_re[q], io, in.ld_psi, S.Ng, ns, ctx->kp_pr[q], ns, 0, st));
-        LRDM_CU(launch_kp_copy(fp64, in.psi_im[q], io, in.ld_psi, S.Ng, ns, ctx->kp_pi[q], ns, 0, st));
-        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_Xr[q]), xc * csz));
-        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_Xi[q]), xc * csz));
-        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_Yr[q]), (size_t)S.kmax * mat * csz));
-        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_Yi[q]), (size_t)S.kmax * mat * csz));
+        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_C[q]), 2 * npsi * csz, false));
+        LRDM_CU(launch_kp_copy(fp64, in.psi_re[q], io, in.ld_psi, S.Ng, ns, ctx->kp_C[q], 2 * ns, 0, st));
+        LRDM_CU(launch_kp_copy(fp64, in.psi_im[q], io, in.ld_psi, S.Ng, ns, ctx->kp_C[q], 2 * ns, ns, st));
+        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_P[q]), S.xslots * mat2 * csz));
+        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_Y[q]), (size_t)S.kmax * mat2 * csz));
         if (!in.rho)
-          LRDM_CU(launch_kp_density(fp64, ctx->kp_pr[q], ctx->kp_pi[q], ns, ns, S.Ng, ctx->kp_occ[q],
-                                    S.g * ctx->kp_w[q], q == 0, in.rho_floor, ch.rho, st));
+          LRDM_CU(launch_kp_density(fp64, ctx->kp_C[q], static_cast<const char*>(ctx->kp_C[q]) + ns * csz, ns,
+                                    2 * ns, S.Ng, ctx->kp_occ[q], S.g * ctx->kp_w[q], q == 0, in.rho_floor,
+                                    ch.rho, st));
         return LRDM_OK;
       }
       // stacked operand C = [Re Psi, Im Psi] in the layouts of the real contractions
@@ -455,7 +453,7 @@ lrdm_status lrdm_kp_create(lrdm_ctx** out, const lrdm_kpoint_system* sys, const 
 
 lrdm_status lrdm_kp_get_split(lrdm_ctx* ctx, int K, int* split) {
   if (!ctx || !ctx->kp || !split || K < 1 || K > ctx->sys[0].kmax) return LRDM_ERR_INVALID_ARG;
-  *split = is_tc(ctx->opt.prec) ? kp_choose_split(ctx, K) : ctx->kp_nsplit;
+  *split = kp_split(ctx, K);
   return LRDM_OK;
 }
 
