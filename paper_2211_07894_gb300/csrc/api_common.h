@@ -57,6 +57,7 @@ lrdm_status setup_poisson(lrdm_ctx* ctx, SysState& S, cudaStream_t st);
 lrdm_status hartree(lrdm_ctx* ctx, SysState& S, int K, cudaStream_t st);
 // grouped tensor-core launch of ctx->tc_entries (gemm 1: projection, 2: response)
 lrdm_status tc_group(lrdm_ctx* ctx, int gemm, int out_is_io, cudaStream_t st);
+int tc_split(long long items, long long units, int nch, int smax);
 // launch-shape tuner of the tensor-core contractions (options.autotune)
 lrdm_status autotune(lrdm_ctx* ctx, cudaStream_t st);
 void free_ctx(lrdm_ctx* ctx);

@@ -259,36 +259,62 @@ struct DmuArgs {
   int nspin;
   int K;
 };
-__global__ void k_dmu(DmuArgs A, int acc64, double* __restrict__ dmu, double* __restrict__ dmu_out,
-                      int* __restrict__ status) {
-  int k = blockIdx.x;
-  double num = 0.0, den = 0.0;
+// num = sum_s sum_i L_ii X_ii and den = sum_s sum_i L_ii of direction k, valid
+// in thread 0.  FP32 partials (the FP32 and tensor-core modes) are summed and
+// multiplied as FP32 pairs: in FP64 the block's one SM, at two operations a
+// clock, took 13 to 30 us for what is one chain of load latencies.
+__device__ __forceinline__ void trace_sums(const DmuArgs& A, int k, int acc64, double& num, double& den) {
+  __shared__ double sn[32], sd[32];
+  __shared__ Pair32 sh[32];
+  if (!acc64) {
+    Pair32 n{0.f, 0.f}, d{0.f, 0.f};
+    for (int s = 0; s < A.nspin; ++s) {
+      const long long mat = (long long)A.ldx[s] * A.ldx[s];
+      for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
+        const Pair32 l = pair_split(A.L[s][(long long)i * A.ns[s] + i]);
+        const Pair32 x = sum_strided_pair(static_cast<const float*>(A.X[s]) + k * mat + (long long)i * A.ldx[s] + i,
+                                          A.nsplit, A.K * mat);
+        pair_fma(n, l, x);
+        pair_add(d, l);
+      }
+    }
+    num = pair_value(pair_block_sum(n, sh));
+    den = pair_value(pair_block_sum(d, sh));
+    return;
+  }
+  num = den = 0.0;
   for (int s = 0; s < A.nspin; ++s) {
-    long long mat = (long long)A.ldx[s] * A.ldx[s];
+    const long long mat = (long long)A.ldx[s] * A.ldx[s];
     for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
-      const long long o = k * mat + (long long)i * A.ldx[s] + i;
-      const double x = acc64 ? sum_strided(static_cast<const double*>(A.X[s]) + o, A.nsplit, A.K * mat)
-                             : sum_strided(static_cast<const float*>(A.X[s]) + o, A.nsplit, A.K * mat);
-      double l = A.L[s][(long long)i * A.ns[s] + i];
+      const double x = sum_strided(static_cast<const double*>(A.X[s]) + k * mat + (long long)i * A.ldx[s] + i,
+                                   A.nsplit, A.K * mat);
+      const double l = A.L[s][(long long)i * A.ns[s] + i];
       num += l * x;
       den += l;
     }
   }
-  __shared__ double sn[32], sd[32];
   for (int o = 16; o > 0; o >>= 1) {
     num += __shfl_xor_sync(0xffffffffu, num, o);
     den += __shfl_xor_sync(0xffffffffu, den, o);
   }
-  int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) { sn[wid] = num; sd[wid] = den; }
+  const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31) == 0) { sn[wid] = num; sd[wid] = den; }
   __syncthreads();
   if (threadIdx.x == 0) {
-    double a = 0, b = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { a += sn[w]; b += sd[w]; }
-    double m = b != 0.0 ? a / b : 0.0;
+    num = den = 0.0;
+    for (int w = 0; w < nw; ++w) { num += sn[w]; den += sd[w]; }
+  }
+}
+
+__global__ void k_dmu(DmuArgs A, int acc64, double* __restrict__ dmu, double* __restrict__ dmu_out,
+                      int* __restrict__ status) {
+  double num, den;
+  trace_sums(A, blockIdx.x, acc64, num, den);
+  if (threadIdx.x == 0) {
+    const double m = den != 0.0 ? num / den : 0.0;
     if (!isfinite(m)) { atomicOr(status, STATUS_NONFINITE); }
-    dmu[k] = m;
-    if (dmu_out) dmu_out[k] = m;
+    dmu[blockIdx.x] = m;
+    if (dmu_out) dmu_out[blockIdx.x] = m;
   }
 }
 
@@ -388,26 +414,9 @@ __global__ void k_loewner_scale_tc(const float* __restrict__ X, int nsplit, int 
 // Backward trace terms T_k = sum_s sum_m L_mm Gbar_k,mm (the adjoint of the
 // mu' constraint) -- same reduction as k_dmu without the division.
 __global__ void k_trace_bar(DmuArgs A, int acc64, double* __restrict__ tbar) {
-  int k = blockIdx.x;
-  double num = 0.0;
-  for (int s = 0; s < A.nspin; ++s) {
-    long long mat = (long long)A.ldx[s] * A.ldx[s];
-    for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
-      const long long o = k * mat + (long long)i * A.ldx[s] + i;
-      const double x = acc64 ? sum_strided(static_cast<const double*>(A.X[s]) + o, A.nsplit, A.K * mat)
-                             : sum_strided(static_cast<const float*>(A.X[s]) + o, A.nsplit, A.K * mat);
-      num += A.L[s][(long long)i * A.ns[s] + i] * x;
-    }
-  }
-  __shared__ double sn[32];
-  for (int o = 16; o > 0; o >>= 1) num += __shfl_xor_sync(0xffffffffu, num, o);
-  if ((threadIdx.x & 31) == 0) sn[threadIdx.x >> 5] = num;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += sn[w];
-    tbar[k] = a;
-  }
+  double num, den;
+  trace_sums(A, blockIdx.x, acc64, num, den);
+  if (threadIdx.x == 0) tbar[blockIdx.x] = num;
 }
 
 // One block per state i of channel s:
@@ -706,14 +715,14 @@ static DmuArgs dmu_args(const SysState& S, const void* const* X, int K) {
 cudaError_t launch_dmu(const SysState& S, const void* const* Xparts, int K, int acc_fp64,
                        double* dmu, double* dmu_out, int* status, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  k_dmu<<<K, 1024, 0, st>>>(dmu_args(S, Xparts, K), acc_fp64, dmu, dmu_out, status);
+  k_dmu<<<K, acc_fp64 ? 256 : 1024, 0, st>>>(dmu_args(S, Xparts, K), acc_fp64, dmu, dmu_out, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_trace_bar(const SysState& S, const void* const* Gparts, int K, int acc_fp64,
                              double* tbar, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  k_trace_bar<<<K, 1024, 0, st>>>(dmu_args(S, Gparts, K), acc_fp64, tbar);
+  k_trace_bar<<<K, acc_fp64 ? 256 : 1024, 0, st>>>(dmu_args(S, Gparts, K), acc_fp64, tbar);
   return cudaGetLastError();
 }
 

@@ -16,42 +16,57 @@
 namespace lrdm {
 namespace {
 
-// mu'_k over all k-points (one block of 1024 threads per direction over all
-// (point, state) pairs: a chain of dependent load latencies otherwise).
-__global__ void __launch_bounds__(1024) k_kp_dmu(KpDmuArgs A, double* __restrict__ dmu,
-                                                double* __restrict__ dmu_out) {
+// mu'_k over all k-points: one block per direction over all (point, state)
+// pairs; FP32 partials summed and multiplied as FP32 pairs (FP64 sums bound the
+// block's one SM).
+__global__ void __launch_bounds__(1024) k_kp_dmu(const __grid_constant__ KpDmuArgs A, double* __restrict__ dmu,
+                                                 double* __restrict__ dmu_out) {
+  __shared__ double sn[32], sd[32];
+  __shared__ Pair32 sh[32];
   const int k = blockIdx.x;
-  double num = 0.0, den = 0.0;
   const long long mat = (long long)A.ld * A.ld;
+  double num = 0.0, den = 0.0;
+  Pair32 n{0.f, 0.f}, d{0.f, 0.f};
   for (int e = threadIdx.x; e < A.nk * A.ns; e += blockDim.x) {
     const int kp = e / A.ns, i = e - kp * A.ns;
-    const double wk = A.kw[kp];
+    const double l = A.kw[kp] * A.L[kp][(long long)i * A.ns + i];
     const long long o = k * mat + (long long)i * A.ld + i, o2 = o + (long long)A.ns * A.ld + A.ns;
-    const double x = A.fp64 ? sum_strided(static_cast<const double*>(A.P[kp]) + o, A.nsplit, A.K * mat) +
-                                  sum_strided(static_cast<const double*>(A.P[kp]) + o2, A.nsplit, A.K * mat)
-                            : sum_strided(static_cast<const float*>(A.P[kp]) + o, A.nsplit, A.K * mat) +
-                                  sum_strided(static_cast<const float*>(A.P[kp]) + o2, A.nsplit, A.K * mat);
-    const double l = A.L[kp][(long long)i * A.ns + i];
-    num += wk * l * x;
-    den += wk * l;
-  }
-  __shared__ double sn[32], sd[32];
-  for (int o = 16; o > 0; o >>= 1) {
-    num += __shfl_xor_sync(0xffffffffu, num, o);
-    den += __shfl_xor_sync(0xffffffffu, den, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sn[threadIdx.x >> 5] = num;
-    sd[threadIdx.x >> 5] = den;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      a += sn[w];
-      b += sd[w];
+    if (A.fp64) {
+      const double* P = static_cast<const double*>(A.P[kp]);
+      num += l * (sum_strided(P + o, A.nsplit, A.K * mat) + sum_strided(P + o2, A.nsplit, A.K * mat));
+      den += l;
+    } else {
+      const float* P = static_cast<const float*>(A.P[kp]);
+      Pair32 x = sum_strided_pair(P + o, A.nsplit, A.K * mat);
+      pair_add(x, sum_strided_pair(P + o2, A.nsplit, A.K * mat));
+      const Pair32 lp = pair_split(l);
+      pair_fma(n, lp, x);
+      pair_add(d, lp);
     }
-    const double v = b != 0.0 ? a / b : 0.0;
+  }
+  if (A.fp64) {
+    for (int o = 16; o > 0; o >>= 1) {
+      num += __shfl_xor_sync(0xffffffffu, num, o);
+      den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      sn[threadIdx.x >> 5] = num;
+      sd[threadIdx.x >> 5] = den;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      num = den = 0.0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        num += sn[w];
+        den += sd[w];
+      }
+    }
+  } else {
+    num = pair_value(pair_block_sum(n, sh));
+    den = pair_value(pair_block_sum(d, sh));
+  }
+  if (threadIdx.x == 0) {
+    const double v = den != 0.0 ? num / den : 0.0;
     dmu[k] = v;
     if (dmu_out) dmu_out[k] = v;
   }
@@ -128,102 +143,157 @@ __global__ void k_kp_copy(const void* __restrict__ src, int io, int ld, long lon
 }
 
 // M'' at [k][j][i] (i fastest) for i <= j < 2 ns: c_ij M_ij with c = 2 off the
-// diagonal; zero elsewhere (padding included).  One thread per four columns.
-// P (both triangles written by GEMM1) and L are symmetric, so every read
-// takes the entry whose column follows i: consecutive threads read
-// consecutive addresses.
-__global__ void k_kp_scale_tc(const float* __restrict__ P, int nsplit, int K, int ns, int ld,
-                              const double* __restrict__ L, const double* __restrict__ dmu, int layout,
-                              void* __restrict__ out, __nv_bfloat16* __restrict__ out_lo) {
+// diagonal; zero elsewhere (padding included).  One thread per four columns of
+// a row, looping over the directions so that L is read and split into an FP32
+// pair once; P (both triangles written by GEMM1) and L are symmetric, so every
+// read takes the entry whose column follows i.  Sums and products as FP32
+// pairs (about 2^-47; the stored operand keeps 16 bits): in FP64, five
+// operations an entry, the kernel was bound by the FP64 pipe: 48^3, 512
+// complex states, K = 8: 187 us a point, now 62 (59 MB to move).
+__global__ void __launch_bounds__(128) k_kp_scale_tc(const float* __restrict__ P, int nsplit, int K, int ns,
+                                                     int ld, const double* __restrict__ L,
+                                                     const double* __restrict__ dmu, int layout,
+                                                     void* __restrict__ out, __nv_bfloat16* __restrict__ out_lo) {
   const int c0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int j = blockIdx.y;
-  const int k = blockIdx.z;
   if (c0 >= ld) return;
-  const long long mat = (long long)ld * ld;
-  const long long tot = (long long)K * mat;
-  const float* Pk = P + (long long)k * mat;
-  auto Pat = [&](int r, int c) {               // P[r][c] summed over the row ranges
-    double x = 0.0;
-    for (int p = 0; p < nsplit; ++p) x += (double)Pk[(long long)p * tot + (long long)r * ld + c];
-    return x;
-  };
+  const long long mat = (long long)ld * ld, tot = (long long)K * mat;
   const int n2 = 2 * ns;
-  float v[4];
+  const int b = j < ns ? j : j - ns;
+  // per column: the two entries of P that make it (r1 + sg r2), L as a pair
+  // (0 where the entry is zero), the diagonal's FP64 L
+  Pair32 l[4];
+  long long o1[4], o2[4];
+  float sg[4];
+  double ld64 = 0.0;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const int i = c0 + e;
-    double m = 0.0;
-    if (i <= j && j < n2) {
-      const int a = i < ns ? i : i - ns, b = j < ns ? j : j - ns;
-      const double l = L[(long long)b * ns + a];
-      if ((i < ns) == (j < ns)) {              // diagonal blocks: Re Gamma_ab = L_ab (P11 + P22 - mu')
-        const double xr = Pat(b, a) + Pat(ns + b, ns + a);
-        m = l * (xr - (a == b ? dmu[k] : 0.0));
-      } else {                                 // i in block 0, j in block 1: Im Gamma_ab = L_ab (P12 - P21)
-        const double xi = Pat(ns + b, a) - Pat(b, ns + a);
-        m = l * xi;
-      }
-      if (i < j) m *= 2.0;
+    const int a = i < ns ? i : i - ns;
+    l[e] = Pair32{0.f, 0.f};
+    o1[e] = o2[e] = 0;
+    sg[e] = 1.f;
+    if (i > j || j >= n2) continue;
+    const double x = L[(long long)b * ns + a];
+    const double c = i < j ? 2.0 * x : x;
+    l[e].s = (float)c;
+    l[e].c = (float)(c - (double)l[e].s);
+    if (i == j) ld64 = x;
+    if ((i < ns) == (j < ns)) {              // diagonal blocks: Re Gamma_ab = L_ab (P11 + P22 - mu')
+      o1[e] = (long long)b * ld + a;
+      o2[e] = (long long)(ns + b) * ld + ns + a;
+    } else {                                 // i in block 0, j in block 1: Im Gamma_ab = L_ab (P12 - P21)
+      o1[e] = (long long)(ns + b) * ld + a;
+      o2[e] = (long long)b * ld + ns + a;
+      sg[e] = -1.f;
     }
-    v[e] = (float)m;
   }
-  const long long o = ((long long)k * ld + j) * ld + c0;
-  if (layout == 1) {
-    float4 t;
-    t.x = tf32_rna(v[0]);
-    t.y = tf32_rna(v[1]);
-    t.z = tf32_rna(v[2]);
-    t.w = tf32_rna(v[3]);
-    *reinterpret_cast<float4*>(static_cast<float*>(out) + o) = t;
-  } else {
-    const __nv_bfloat162 h01 = __floats2bfloat162_rn(v[0], v[1]);
-    const __nv_bfloat162 h23 = __floats2bfloat162_rn(v[2], v[3]);
-    const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
-    const __nv_bfloat162 l01 = __floats2bfloat162_rn(v[0] - f01.x, v[1] - f01.y);
-    const __nv_bfloat162 l23 = __floats2bfloat162_rn(v[2] - f23.x, v[3] - f23.y);
-    uint2 hw, lw;
-    hw.x = *reinterpret_cast<const uint32_t*>(&h01);
-    hw.y = *reinterpret_cast<const uint32_t*>(&h23);
-    lw.x = *reinterpret_cast<const uint32_t*>(&l01);
-    lw.y = *reinterpret_cast<const uint32_t*>(&l23);
-    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + o) = hw;
-    *reinterpret_cast<uint2*>(out_lo + o) = lw;
+  const bool any = c0 <= j && j < n2;
+  // all four columns on or above the diagonal, in one block of columns:
+  // 16-byte loads of both entries (ld is a multiple of 4)
+  const bool quad = c0 + 3 <= j && j < n2 && ns % 4 == 0;
+#pragma unroll 2
+  for (int k = 0; k < K; ++k) {
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (any) {
+      const float* Pk = P + (long long)k * mat;
+      Pair32 xs[4];
+      for (int p = 0; p < nsplit; ++p) {
+        float y1[4], y2[4];
+        if (quad) {
+          *reinterpret_cast<float4*>(y1) = *reinterpret_cast<const float4*>(Pk + p * tot + o1[0]);
+          *reinterpret_cast<float4*>(y2) = *reinterpret_cast<const float4*>(Pk + p * tot + o2[0]);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            y1[e] = Pk[p * tot + o1[e]];
+            y2[e] = Pk[p * tot + o2[e]];
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          if (p == 0) xs[e] = Pair32{y1[e], 0.f};
+          else pair_add(xs[e], Pair32{y1[e], 0.f});
+          pair_add(xs[e], Pair32{sg[e] * y2[e], 0.f});
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (c0 + e > j) continue;
+        const Pair32 x = xs[e];
+        if (c0 + e == j) {
+          v[e] = (float)(ld64 * ((double)x.s + (double)x.c - (j < n2 ? dmu[k] : 0.0)));
+        } else {
+          const float q = __fmul_rn(l[e].s, x.s);
+          const float qe = __fmaf_rn(l[e].c, x.s, __fmaf_rn(l[e].s, x.c, __fmaf_rn(l[e].s, x.s, -q)));
+          v[e] = __fadd_rn(q, qe);
+        }
+      }
+    }
+    const long long o = ((long long)k * ld + j) * ld + c0;
+    if (layout == 1) {
+      float4 t;
+      t.x = tf32_rna(v[0]);
+      t.y = tf32_rna(v[1]);
+      t.z = tf32_rna(v[2]);
+      t.w = tf32_rna(v[3]);
+      *reinterpret_cast<float4*>(static_cast<float*>(out) + o) = t;
+    } else {
+      const __nv_bfloat162 h01 = __floats2bfloat162_rn(v[0], v[1]);
+      const __nv_bfloat162 h23 = __floats2bfloat162_rn(v[2], v[3]);
+      const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
+      const __nv_bfloat162 l01 = __floats2bfloat162_rn(v[0] - f01.x, v[1] - f01.y);
+      const __nv_bfloat162 l23 = __floats2bfloat162_rn(v[2] - f23.x, v[3] - f23.y);
+      uint2 hw, lw;
+      hw.x = *reinterpret_cast<const uint32_t*>(&h01);
+      hw.y = *reinterpret_cast<const uint32_t*>(&h23);
+      lw.x = *reinterpret_cast<const uint32_t*>(&l01);
+      lw.y = *reinterpret_cast<const uint32_t*>(&l23);
+      *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + o) = hw;
+      *reinterpret_cast<uint2*>(out_lo + o) = lw;
+    }
   }
 }
 
-// f = sum_kappa part_kappa - v, FP64 sum of the FP32 contributions
-__global__ void k_kp_sum(KpSumArgs A, const void* __restrict__ v, int io, long long n,
+// The points' FP32 contributions at o, added as an FP32 pair (in FP64 the
+// conversions and additions bound the kernel: 24 us at 48^3, 4 points, K = 8).
+__device__ __forceinline__ Pair32 kp_parts(const KpSumArgs& A, long long o) {
+  Pair32 d{A.part[0][o], 0.f};
+  for (int q = 1; q < A.nk; ++q) pair_add(d, Pair32{A.part[q][o], 0.f});
+  return d;
+}
+
+// f = sum_kappa part_kappa - v
+__global__ void k_kp_sum(const __grid_constant__ KpSumArgs A, const void* __restrict__ v, int io, long long n,
                          void* __restrict__ f) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x) {
-    double d = 0.0;
-    for (int q = 0; q < A.nk; ++q) d += (double)A.part[q][e];
-    if (io == LRDM_DTYPE_F64)
-      static_cast<double*>(f)[e] = d - static_cast<const double*>(v)[e];
-    else
-      static_cast<float*>(f)[e] = (float)(d - (double)static_cast<const float*>(v)[e]);
+    Pair32 d = kp_parts(A, e);
+    if (io == LRDM_DTYPE_F64) {
+      static_cast<double*>(f)[e] = (double)d.s + (double)d.c - static_cast<const double*>(v)[e];
+    } else {
+      pair_add(d, Pair32{-static_cast<const float*>(v)[e], 0.f});
+      static_cast<float*>(f)[e] = __fadd_rn(d.s, d.c);
+    }
   }
 }
 
-// out[k][r] (compute type, row stride ld) = sum_kappa part_kappa[k][r]
-// (A given: FP32 contributions) or drho[k][r] (FP64 accumulator); zero for
-// N_g <= r < ld.
-__global__ void k_kp_collect(KpSumArgs A, int use_parts, const double* __restrict__ drho, long long Ng,
-                             long long ld, long long tot, void* __restrict__ out, int fp64) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long k = e / ld, r = e - k * ld;
-    double d = 0.0;
-    if (r < Ng) {
-      const long long o = k * Ng + r;
-      if (use_parts)
-        for (int q = 0; q < A.nk; ++q) d += (double)A.part[q][o];
-      else
-        d = drho[o];
-    }
-    if (fp64) static_cast<double*>(out)[e] = d;
-    else static_cast<float*>(out)[e] = (float)d;
+// out[k][r] (compute type, row stride ld; k = blockIdx.y) = sum_kappa
+// part_kappa[k][r] (use_parts: FP32 contributions) or drho[k][r] (FP64
+// accumulator); zero for N_g <= r < ld.
+__global__ void k_kp_collect(const __grid_constant__ KpSumArgs A, int use_parts,
+                             const double* __restrict__ drho, long long Ng, long long ld,
+                             void* __restrict__ out, int fp64) {
+  const long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x, k = blockIdx.y;
+  if (r >= ld) return;
+  Pair32 d{0.f, 0.f};
+  double d64 = 0.0;
+  if (r < Ng) {
+    if (use_parts) d = kp_parts(A, k * Ng + r);
+    else d64 = drho[k * Ng + r];
   }
+  if (fp64) static_cast<double*>(out)[k * ld + r] = use_parts ? (double)d.s + (double)d.c : d64;
+  else static_cast<float*>(out)[k * ld + r] = use_parts ? __fadd_rn(d.s, d.c) : (float)d64;
 }
 
 inline unsigned kp_grid(long long n, int threads) {
@@ -236,7 +306,7 @@ inline unsigned kp_grid(long long n, int threads) {
 
 cudaError_t launch_kp_dmu(const KpDmuArgs& A, double* dmu, double* dmu_out, cudaStream_t st) {
   if (A.K == 0) return cudaSuccess;
-  k_kp_dmu<<<A.K, 1024, 0, st>>>(A, dmu, dmu_out);
+  k_kp_dmu<<<A.K, A.fp64 ? 256 : 1024, 0, st>>>(A, dmu, dmu_out);
   return cudaGetLastError();
 }
 
@@ -284,7 +354,7 @@ cudaError_t launch_kp_copy(int fp64, const void* src, int io, int ld, long long 
 cudaError_t launch_kp_scale_tc(const float* P, int nsplit, int K, int ns, int ld, const double* L,
                                const double* dmu, int layout, void* out, void* out_lo, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  dim3 grid((unsigned)((ld / 4 + 127) / 128), (unsigned)ld, (unsigned)K);
+  dim3 grid((unsigned)((ld / 4 + 127) / 128), (unsigned)ld);
   k_kp_scale_tc<<<grid, 128, 0, st>>>(P, nsplit, K, ns, ld, L, dmu, layout, out,
                                       static_cast<__nv_bfloat16*>(out_lo));
   return cudaGetLastError();
@@ -293,10 +363,10 @@ cudaError_t launch_kp_scale_tc(const float* P, int nsplit, int K, int ns, int ld
 cudaError_t launch_kp_collect(const KpSumArgs* A, const double* drho, int K, long long Ng, long long ld,
                               void* out, int fp64, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  const long long tot = (long long)K * ld;
   KpSumArgs a{};
   if (A) a = *A;
-  k_kp_collect<<<kp_grid(tot, 256), 256, 0, st>>>(a, A ? 1 : 0, drho, Ng, ld, tot, out, fp64);
+  const dim3 grid((unsigned)((ld + 255) / 256), (unsigned)K);
+  k_kp_collect<<<grid, 256, 0, st>>>(a, A ? 1 : 0, drho, Ng, ld, out, fp64);
   return cudaGetLastError();
 }
 

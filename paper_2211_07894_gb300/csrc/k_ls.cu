@@ -84,14 +84,6 @@ __global__ void __launch_bounds__(256) k_gram(const T* __restrict__ F, const T* 
 // (all with the elimination; 2e-15 with the Jacobi rotations).
 constexpr long long LS_N32 = 65536;
 
-__device__ __forceinline__ Pair32 warp_sum(Pair32 a) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const Pair32 b{__shfl_xor_sync(0xffffffffu, a.s, o), __shfl_xor_sync(0xffffffffu, a.c, o)};
-    pair_add(a, b);
-  }
-  return a;
-}
 // a += x . y over four points.  The four products are summed first and the
 // rounding errors of products and of sums kept apart until the end: a square's
 // error word ends in fixed bits (x^2 = 1 mod 8), and dropping them one product
@@ -234,7 +226,7 @@ __device__ __forceinline__ void gr_task(const float* __restrict__ F, const float
       for (int i = 0; i < NA; ++i)
 #pragma unroll
         for (int j = DIAG ? i : 0; j < NB; ++j) {
-          const Pair32 a = warp_sum(acc[i][j]);
+          const Pair32 a = pair_warp_sum(acc[i][j]);
           if (lane == 0) out[4 * i + j] = (fresh ? 0.0 : out[4 * i + j]) + ((double)a.s + (double)a.c);
         }
     } else {
@@ -607,11 +599,6 @@ __device__ __forceinline__ void axpy2(Pair32& a, float h, float l, float x) {
   two_sum(a.s, p, a.s, r);
   a.c = __fadd_rn(a.c, __fadd_rn(e, r));
 }
-__device__ __forceinline__ Pair32 split2(double x) {
-  const float h = (float)x;
-  return Pair32{h, (float)(x - (double)h)};
-}
-
 // The same for FP32 data, in compensated FP32 (2 K fma a point in FP64 bound
 // it to the FP64 rate).  Two points a thread, the K loop unrolled for loads in
 // flight; what is the same for all threads is made once a block (a division
@@ -634,7 +621,7 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
   __shared__ int se;
   __shared__ double sw[8];
   if (threadIdx.x < KMAX_LIMIT + UB) {
-    const Pair32 p = split2(threadIdx.x < K ? coef[threadIdx.x] : 0.0);
+    const Pair32 p = pair_split(threadIdx.x < K ? coef[threadIdx.x] : 0.0);
     a[threadIdx.x] = make_float2(p.s, p.c);
   }
   if (threadIdx.x == 128) {
@@ -643,7 +630,7 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
     se = ms > 0.0 && isfinite(ms) ? max(-120, min(120, -ilogb(ms) / 2)) : 0;
   }
   __syncthreads();
-  const Pair32 al = split2(alpha);
+  const Pair32 al = pair_split(alpha);
   const int e = se;
   const float sc = __int_as_float((127 + e) << 23);
   double acc = 0.0;
@@ -741,7 +728,7 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
       if (RHO) rho[r] = out;
     }
   }
-  sq = warp_sum(sq);
+  sq = pair_warp_sum(sq);
   if (__any_sync(0xffffffffu, acc != 0.0))
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = acc + ldexp((double)sq.s + (double)sq.c, -2 * e);

@@ -238,8 +238,8 @@ lrdm_status setup_system(lrdm_ctx* ctx, int idx, const lrdm_system& in, cudaStre
   const int accsz = fp64 ? 8 : 4;
   // the X / G buffers hold several grid-row partials of a k_max-direction call
   // while they stay within 512 MB per channel, so that few tiles (a small
-  // subspace) can split their grid reduction: up to 8 on the tensor cores, on
-  // the CUDA cores the count simt_split takes (row-sharded: one per rank)
+  // subspace) can split their grid reduction (CUDA cores: the count simt_split
+  // takes; row-sharded: one per rank)
   S.xslots = S.kmax;
   {
     size_t ldmax = 0;
@@ -247,7 +247,12 @@ lrdm_status setup_system(lrdm_ctx* ctx, int idx, const lrdm_system& in, cudaStre
       ldmax = std::max(ldmax, (size_t)(is_tc(prec) ? S.ch[c].ns_pad : S.ch[c].ns));
     const size_t per = (size_t)S.kmax * ldmax * ldmax * accsz;
     const int room = (int)std::min<size_t>(64, std::max<size_t>(1, (512ull << 20) / per));
-    if (is_tc(prec)) S.xslots = std::min(8, room) * S.kmax;
+    if (is_tc(prec)) {
+      // up to 8 calls' worth, or 32 slots where those are small (one direction
+      // of a small subspace: K = 1 calls then split as far as tc_split wants)
+      S.xslots = std::min(8, room) * S.kmax;
+      while (S.xslots < 32 && (size_t)(S.xslots + 1) * ldmax * ldmax * accsz <= (64ull << 20)) ++S.xslots;
+    }
     else if (!ctx->rows) S.xslots = simt_split(fp64, S.ch[0].ns, S.Ng, S.kmax, room * S.kmax) * S.kmax;
   }
   for (int c = 0; c < in.nspin; ++c) {
@@ -368,15 +373,27 @@ lrdm_status tc_group(lrdm_ctx* ctx, int gemm, int out_is_io, cudaStream_t st) {
   return from_cuda(e);
 }
 
-// Grid-row ranges of the tensor-core GEMM1 for K directions of system s.
-// The work items (tiles x directions x ranges) are of equal size, so the
-// launch time follows the number of waves over the SMs: the count that fills
-// the last wave best (by more than half a percent over a smaller count), with
-// at most 8 ranges, nsplit * K <= the X buffer's direction slots (k_max, or
-// up to 8 k_max for small subspaces) and at least 64 stages of the reduction
-// per range.  1 at the
-// benchmark's K = 16 (4352 items, 0.987 of 29 waves); 5 at K = 1 there
-// (1360 items, 0.994 of 9 waves, against 0.895 for 1-4 ranges).
+// Row ranges of a projection launch of `items` equal work items on `units` grid
+// units, nch stages of the reduction each: the launch takes as many waves as
+// there are items per unit, an item nch / sp stages and about 100 stages'
+// worth of start, last flush and tile store; the smallest count within half a
+// percent of the least, at least 128 stages a range.  48^3 / 512, K = 1 (3 items
+// for 76 pairs): 25 ranges, 228 -> 112 us against the former limit of 8; K = 2:
+// 12, 231 -> 180 us; K = 8 (24 items): 3; 96^3 / 4096, K = 16: 1.
+int tc_split(long long items, long long units, int nch, int smax) {
+  auto cost = [&](long long sp) {
+    return (double)((items * sp + units - 1) / units) * ((double)nch / (double)sp + 100.0);
+  };
+  double low = cost(1);
+  smax = std::min(smax, nch / 128);
+  for (int sp = 2; sp <= smax; ++sp) low = std::min(low, cost(sp));
+  for (int sp = 1; sp <= smax; ++sp)
+    if (cost(sp) <= 1.005 * low) return sp;
+  return 1;
+}
+
+// Grid-row ranges of GEMM1 for K directions of system s (tensor cores: the
+// count of tc_split, nsplit * K at most the X buffer's direction slots).
 int choose_split(lrdm_ctx* ctx, int s, int K) {
   const SysState& S = ctx->sys[s];
   if (K <= 0 || ctx->rows) return 1;
@@ -390,20 +407,7 @@ int choose_split(lrdm_ctx* ctx, int s, int K) {
       (long long)(pair ? pr.ntiles_p : wide ? pr.ntiles_w : pr.ntiles) * ((K + dpt - 1) / dpt);
   // work units of the persistent grid: SMs, or CTA pairs for the pair tiles
   const long long sms = pair ? tc_pair_units(ctx->opt.prec) : ctx->sm_count > 0 ? ctx->sm_count : 148;
-  int smax = S.xslots / K;
-  if (smax > 8) smax = 8;
-  if (smax > pr.nch / 64) smax = pr.nch / 64;
-  int best = 1;
-  double best_fill = 0.0;
-  for (int sp = 1; sp <= smax; ++sp) {
-    const long long n = items * sp;
-    const double fill = (double)n / (double)(((n + sms - 1) / sms) * sms);
-    if (fill > best_fill + 0.005) {
-      best_fill = fill;
-      best = sp;
-    }
-  }
-  return best;
+  return tc_split(items, sms, pr.nch, S.xslots / K);
 }
 
 TcEntry tc_entry(lrdm_ctx* ctx, int s, int c, int K) {

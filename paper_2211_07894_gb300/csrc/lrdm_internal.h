@@ -39,6 +39,40 @@ __device__ __forceinline__ void pair_add(Pair32& a, const Pair32& b) {
   two_sum(a.s, b.s, a.s, r);
   a.c = __fadd_rn(a.c, __fadd_rn(b.c, r));
 }
+__device__ __forceinline__ Pair32 pair_split(double x) {
+  const float h = (float)x;
+  return Pair32{h, (float)(x - (double)h)};
+}
+// a += x y (both pairs; relative error about 2^-46)
+__device__ __forceinline__ void pair_fma(Pair32& a, const Pair32& x, const Pair32& y) {
+  const float p = __fmul_rn(x.s, y.s);
+  const float e = __fmaf_rn(x.s, y.c, __fmaf_rn(x.c, y.s, __fmaf_rn(x.s, y.s, -p)));
+  pair_add(a, Pair32{p, e});
+}
+__device__ __forceinline__ Pair32 pair_warp_sum(Pair32 a) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    pair_add(a, Pair32{__shfl_xor_sync(0xffffffffu, a.s, o), __shfl_xor_sync(0xffffffffu, a.c, o)});
+  return a;
+}
+__device__ __forceinline__ double pair_value(const Pair32& a) { return (double)a.s + (double)a.c; }
+// Sum over the block (all threads call it), valid in every thread of warp 0.
+__device__ __forceinline__ Pair32 pair_block_sum(Pair32 a, Pair32* sh) {
+  a = pair_warp_sum(a);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
+  __syncthreads();
+  Pair32 r{0.f, 0.f};
+  if (threadIdx.x < (blockDim.x >> 5)) r = sh[threadIdx.x];
+  if (threadIdx.x < 32) r = pair_warp_sum(r);
+  __syncthreads();
+  return r;
+}
+__device__ __forceinline__ Pair32 sum_strided_pair(const float* __restrict__ p, int n, long long stride) {
+  Pair32 x{p[0], 0.f};
+#pragma unroll 8
+  for (int i = 1; i < n; ++i) pair_add(x, Pair32{p[i * stride], 0.f});
+  return x;
+}
 // Sum of n values p[0], p[stride], ..: FP64 data in FP64, FP32 data as an FP32
 // pair (48 bits; one FP64 addition and one conversion a value cost 128 FP32
 // operations on GB300).
@@ -49,10 +83,7 @@ __device__ __forceinline__ double sum_strided(const double* __restrict__ p, int 
   return x;
 }
 __device__ __forceinline__ double sum_strided(const float* __restrict__ p, int n, long long stride) {
-  Pair32 x{p[0], 0.f};
-#pragma unroll 4
-  for (int i = 1; i < n; ++i) pair_add(x, Pair32{p[i * stride], 0.f});
-  return (double)x.s + (double)x.c;
+  return pair_value(sum_strided_pair(p, n, stride));
 }
 
 // NVTX range for the profilers' timelines (one per API call and per phase of

@@ -59,9 +59,7 @@ lrdm_status solve_mu_kp_host(const std::vector<std::vector<double>>& eps, const 
 // forward passes a = w dV and factor g; the adjoint a = fbar and factor w g
 // (the map is self-adjoint, the same traceless projection applies).
 // Grid-row ranges of the tensor-core projection for K directions over all
-// k-points: the fewest ranges (up to the P buffers' capacity, at least 64
-// stages each) whose work items fill the persistent grid's waves to 90 %,
-// else the best fill.
+// k-points (tc_split; up to the P buffers' capacity).
 int kp_choose_split(lrdm_ctx* ctx, int K) {
   const bool pair = ctx->tune.g1_nb == G1_PAIR;
   // work units of the persistent grid: SMs, or CTA pairs for the pair tiles
@@ -75,19 +73,7 @@ int kp_choose_split(lrdm_ctx* ctx, int K) {
     per += (long long)(pair ? pr.ntiles_p : wide ? pr.ntiles_w : pr.ntiles) * ((K + dpt - 1) / dpt);
     nch = std::min(nch, pr.nch);
   }
-  int best = 1;
-  double best_fill = 0.0;
-  for (int s = 1; s <= ctx->kp_split_cap && nch / s >= 64; ++s) {
-    const long long items = per * s;
-    const long long waves = (items + sms - 1) / sms;
-    const double fill = (double)items / (double)(waves * sms);
-    if (fill > best_fill + 1e-9) {
-      best_fill = fill;
-      best = s;
-    }
-    if (fill >= 0.9) break;
-  }
-  return best;
+  return tc_split(per, sms, nch, ctx->kp_split_cap);
 }
 
 // Grid-row ranges of the projection for K directions.
