@@ -1309,23 +1309,50 @@ __global__ void __launch_bounds__(G1_THREADS, 1)
 }
 
 // ===========================================================================
-// GEMM1 on CTA pairs (cta_group::2): 256 x 256 tiles, one direction
+// GEMM1 on CTA pairs (cta_group::2)
 // ===========================================================================
 //
-// A cluster of two CTAs on neighbouring SMs computes one 256 x 256 tile
-// (I2, J) of X_k, I2 <= J in 256-state blocks, with M = 256 pair MMAs: CTA r
-// of the pair loads (by TMA) and weights the FP32 Psi^T rows of the 128-state
-// block 2 I2 + r into its own tensor memory (the A rows of the MMA), and loads
-// the bf16 hi / lo (or TF32) Psi^T rows of the 128-state block 2 J + r (its
-// half of the B rows).  One thread of the even CTA issues the MMAs; each CTA's
-// tensor memory receives its 128 rows x 256 columns of the accumulator.  Per
-// SM that halves the B rows loaded and read per MMA, against the 128 x 256
+// A cluster of two CTAs on neighbouring SMs works with M = 256, N = 256 pair
+// MMAs: CTA r of the pair loads (by TMA) and weights the FP32 Psi^T rows of a
+// 128-state block into its own tensor memory (its half of the A rows), and
+// loads the bf16 hi / lo (or TF32) Psi^T rows of a 128-state block of columns
+// (its half of the B rows).  One thread of the even CTA issues the MMAs; each
+// CTA's tensor memory receives its 128 rows x 256 columns of the accumulator.
+// Per SM that halves the B rows loaded and read per MMA, against the 128 x 256
 // single-CTA tile, for the same MMA work.
 //
+// X_k is symmetric: a block (b, c) of it, computed on either side of the
+// diagonal, gives (c, b) too, so the upper triangle is all that is needed.
+// Directions are taken in twos: both CTAs load row block b, CTA r weights it
+// with direction 2 g + r, and the column blocks c0, c1 are any two with (b, c0)
+// and (b, c1) still to be done (g1p_blocks): n (n + 1) / 4 items per two
+// directions for n block rows, rounded up.  256 x 256 tiles of one direction, which also compute the part of their
+// diagonal tiles below it and pad n to an even number, take n (n + 2) / 8 each;
+// they are kept for the last direction of an odd number.  With it and the
+// separate accumulating warps below, against 256 x 256 tiles weighted and
+// accumulated by the same warps (BF16x3 / TF32): 48^3, N_s = 512, K = 8: 594 ->
+// 492 us / 501 -> 408 us; 64^3 / 1024 / 16: 9.49 -> 8.28 ms; 72^3 / 2048 / 12:
+// TF32 29.4 -> 25.7 ms; 40^3 / 384 / 6: 286 -> 137 us.  What binds: BF16x3 runs
+// at the tensor rate under the power limit (1.8 PFLOP/s of MMAs at 64^3); TF32
+// at the shared-memory port (64 KB a stage of 512 clocks).  Both CTAs load the
+// same A rows; multicast of halves to both was slower (BF16x3 2 %, TF32 15 %).
+// N = 128 MMAs with A in TMEM take as long as N = 256, so neither narrower
+// tiles for the odd blocks nor halves of the accumulator pay.
+//
 // Barriers: full[s] (each CTA, its own TMA bytes); ready[s] and acc_empty
-// (even CTA, 16 arrivals: the 8 math warps of both CTAs); empty[s] and
+// (even CTA, 16 arrivals: 8 warps of both CTAs, weighting and accumulating); empty[s] and
 // acc_full (both CTAs, one arrival each from the multicast MMA commit); drain
 // (even CTA).  The reduction is segmented as in k_gemm1_tc.
+
+// Warps 0-7 (warpgroups 0, 1) weight, 8-15 (2, 3) accumulate the segments and
+// store, warp 16 loads, 17 issues the MMAs and owns the TMEM: with the first
+// two in the same warps a segment's end (some 500 clocks) and a tile's stores
+// (13-16 thousand) held up the weighting (48^3, N_s = 512, K = 8: 488 -> 475 us,
+// TF32 419 -> 401 us).  Registers: 640 x 96 at launch = 256 x 40 + 256 x 176 +
+// 128 x 48; per SM sub-partition (five warps) 32 x 480 = 15360 <= 16384.
+constexpr int G1P_THREADS = 640;
+constexpr int G1P_REG_WEIGHT = 40, G1P_REG_ACC = 176, G1P_REG_CTRL = 48;
+static_assert(256 * G1P_REG_WEIGHT + 256 * G1P_REG_ACC + 128 * G1P_REG_CTRL <= G1P_THREADS * 96, "register split");
 
 template <int PREC>
 struct G1PCfg {
@@ -1342,36 +1369,88 @@ struct G1PCfg {
   static constexpr int SC_OFF = B_OFF + SUB * B_CHUNK;
   static constexpr int STRIDE = SC_OFF + 1024;
   static constexpr int SMEM = STAGES * STRIDE + 1024 + 512;
-  static constexpr int SEG = 1024 / (BK * SUB);
-  static constexpr int LAG = STAGES - 1;
+  // Stages per accumulation segment at most; a range's segments are equally
+  // long.  BF16x3: 768 rows take a quarter off the truncation error of 1024 and
+  // cost 1.5 % (512: half, 5 %; an interruption of the MMAs is some 600 clocks);
+  // TF32's own rounding is far above it.
+  static constexpr int SEG = (PREC == LRDM_BF16X3 ? 768 : 1024) / (BK * SUB);
   static constexpr int TX = A_BYTES + SUB * B_CHUNK + BK * SUB * 4;   // TMA bytes per stage and CTA
   static constexpr uint32_t IDESC = ptx::idesc_make(PREC == LRDM_BF16X3 ? 1 : 2, 256, 256);
   static_assert(G1_ACOL + STAGES * SLOT <= 512, "TMEM budget");
   static_assert(SMEM <= 227 * 1024, "shared memory budget");
 };
 
-// Pair item -> slot q, row range `split`, direction k, tile (I2, J): row
-// ranges outermost, then tiles column by column (column J holds I2 = 0..J),
-// directions fastest (the pairs working on one tile stream the same Psi^T
-// rows through L2).
-__device__ __forceinline__ const TcProblem* g1p_item(const G1Params& P, int item, int& q, int& k,
-                                                     int& I2, int& J, int& split) {
-  q = find_slot(P.begin, P.nslot, item);
-  const TcProblem* pr = P.probs + P.pid[q];
-  int idx = item - P.begin[q];
-  const int K = P.K[q];
-  const int per_split = pr->ntiles_p * K;
-  split = idx / per_split;
-  idx -= split * per_split;
-  int t = idx / K;
-  k = idx - t * K;
-  int j = 0;
-  while (t > j) {
-    t -= j + 1;
-    ++j;
+// Item t of the two-direction items of n block rows: row block b and column
+// blocks c0, c1 (c1 == c0: one block only).  The block rows go in groups of
+// four (the last may have r < 4).  Groups P < Q: the r columns of Q in twos for
+// each row of P, and Q's odd last one as the row block against P's four in
+// twos: 2 r items, every block once.  Within a group the 10 blocks (b <= c) are
+// the pairs 00 01 | 11 12 | 22 20 | 33 32 | 30 31; the first three cover r = 3,
+// the first two without 12, 00 without 01 cover r = 2 and r = 1.
+__host__ __device__ inline int g1p_group_items(int r) { return r == 4 ? 5 : r; }
+
+__host__ __device__ inline void g1p_blocks(int n, int t, int& b, int& c0, int& c1) {
+  int Q = 0, r = n < 4 ? n : 4;
+  while (t >= 2 * r * Q + g1p_group_items(r)) {
+    t -= 2 * r * Q + g1p_group_items(r);
+    ++Q;
+    r = n - 4 * Q < 4 ? n - 4 * Q : 4;
   }
-  J = j;
-  I2 = t;
+  if (t < 2 * r * Q) {
+    const int P = t / (2 * r), u = t - P * 2 * r, e = r >> 1;
+    if (u < 4 * e) {
+      b = 4 * P + u / e;
+      c0 = 4 * Q + 2 * (u - u / e * e);
+    } else {
+      b = 4 * Q + r - 1;
+      c0 = 4 * P + 2 * (u - 4 * e);
+    }
+    c1 = c0 + 1;
+    return;
+  }
+  const int u = t - 2 * r * Q;
+  b = u < 4 ? u : 3;
+  c0 = u < 4 ? u : 0;
+  c1 = u == 4 ? 1 : u == 3 ? 2 : u == 2 ? 0 : u + 1 < r ? u + 1 : u;
+  b += 4 * Q;
+  c0 += 4 * Q;
+  c1 += 4 * Q;
+}
+
+// Pair item -> slot q, row range `split`, this CTA's direction k and row block
+// b, column blocks c0, c1; two: an item of two directions.  Row ranges
+// outermost, then the items of two directions, directions fastest (the pairs
+// working on one tile stream the same Psi^T rows through L2), then the last
+// direction's 256 x 256 tiles (I, J), I <= J, column by column.
+struct G1Item {
+  int q, split, k, b, c0, c1;
+  bool two;
+};
+
+__device__ __forceinline__ const TcProblem* g1p_item(const G1Params& P, int item, int rank, G1Item& x) {
+  x.q = find_slot(P.begin, P.nslot, item);
+  const TcProblem* pr = P.probs + P.pid[x.q];
+  int idx = item - P.begin[x.q];
+  const int K = P.K[x.q], G = K >> 1;
+  const int nd = pr->ntiles_d * G, per_split = nd + ((K & 1) ? pr->ntiles_p : 0);
+  x.split = idx / per_split;
+  idx -= x.split * per_split;
+  x.two = idx < nd;
+  if (x.two) {
+    const int t = idx / G;
+    x.k = 2 * (idx - t * G) + rank;
+    g1p_blocks((pr->ns + BM - 1) / BM, t, x.b, x.c0, x.c1);
+  } else {
+    int t = idx - nd, j = 0;
+    while (t > j) {
+      t -= j + 1;
+      ++j;
+    }
+    x.k = K - 1;
+    x.b = 2 * t + rank;
+    x.c0 = 2 * j;
+    x.c1 = 2 * j + 1;                     // (past the end: zero fill, not stored)
+  }
   return pr;
 }
 
@@ -1419,12 +1498,12 @@ __device__ __forceinline__ void g1p_producer(const G1Params& P, uint8_t* smem, c
   for (int item = pair; item < items && ok; item += npairs, ++round) {
     if (align && round > 0 && !ptx::counter_wait_geq(P.sync, round_target(round - 1, items, npairs, 2), ALIGN_NS))
       align = false;
-    int q, k, I2, J, sp;
-    const TcProblem* pr = g1p_item(P, item, q, k, I2, J, sp);
+    G1Item x;
+    const TcProblem* pr = g1p_item(P, item, rank, x);
     int rb, re;
-    g1_range<SUB>(P, pr, q, sp, rb, re);
-    const float* w0 = pr->a + (long long)k * pr->a_stride;
-    const int ia = 2 * I2 + rank, ib = 2 * J + rank;   // 128-state blocks (past the end: zero fill)
+    g1_range<SUB>(P, pr, x.q, x.split, rb, re);
+    const float* w0 = pr->a + (long long)x.k * pr->a_stride;
+    const int ia = x.b, ib = rank ? x.c1 : x.c0;       // 128-state blocks (past the end: zero fill)
     for (int rc = rb; rc < re; ++rc) {
       if (!wait1(&B.empty[s], ph ^ 1, B, P.status)) { ok = false; break; }
       uint8_t* st = smem + s * C::STRIDE;
@@ -1447,9 +1526,9 @@ __device__ __forceinline__ void g1p_producer(const G1Params& P, uint8_t* smem, c
     if (pending[i] >= 0) wait_drain(&B.full[i], (uint32_t)pending[i]);
 }
 
-// The MMA thread's waits on barriers that both CTAs' math warps arrive on:
+// The MMA thread's waits on barriers that both CTAs' warps arrive on:
 // the CTA-scope try_wait (which suspends the thread between polls; the
-// cluster-scope form spins and takes issue slots from the math warps that
+// cluster-scope form spins and takes issue slots from the other warps that
 // share its sub-partition), paired with the default-semantics remote arrive.
 __device__ __forceinline__ bool wait_cl(uint64_t* bar, uint32_t parity, const Bars& B, int* status) {
   return ptx::mbar_wait(bar, parity, B.abort, status, WAIT_NS, STATUS_TIMEOUT);
@@ -1465,15 +1544,15 @@ __device__ __forceinline__ void g1p_mma(const G1Params& P, uint8_t* smem, const 
   uint32_t ph = 0, aph = 0;
   bool ok = true;
   for (int item = pair; item < items && ok; item += npairs) {
-    int q, k, I2, J, sp;
-    const TcProblem* pr = g1p_item(P, item, q, k, I2, J, sp);
+    G1Item x;
+    const TcProblem* pr = g1p_item(P, item, 0, x);
     int rb, re;
-    g1_range<C::SUB>(P, pr, q, sp, rb, re);
+    g1_range<C::SUB>(P, pr, x.q, x.split, rb, re);
     const int nseg = (re - rb + SEG - 1) / SEG;
     for (int sg = 0; sg < nseg && ok; ++sg) {
       if (!wait_cl(&B.acc_empty[0], aph ^ 1, B, P.status)) { ok = false; break; }
       ptx::tc_fence_after();
-      const int r0 = rb + sg * SEG, r1 = min(re, r0 + SEG);
+      const int r0 = rb + (int)((long long)(re - rb) * sg / nseg), r1 = rb + (int)((long long)(re - rb) * (sg + 1) / nseg);
       for (int rc = r0; rc < r1; ++rc) {
         if (!wait_cl(&B.ready[s], ph, B, P.status)) { ok = false; break; }
         ptx::tc_fence_after();
@@ -1491,76 +1570,111 @@ __device__ __forceinline__ void g1p_mma(const G1Params& P, uint8_t* smem, const 
   wait_drain(B.drain, 0);
 }
 
-// Weighting into this CTA's tensor memory, segment accumulation and the tile
-// epilogue (warps 0-7 of both CTAs; warp w serves TMEM lane quarter w % 4 and
-// element half / accumulator column half w / 4).
+// Weighting into this CTA's tensor memory (warps 0-7 of both CTAs: TMEM lane
+// quarter w % 4, element half w / 4).
 template <int PREC>
-__device__ __forceinline__ void g1p_math(const G1Params& P, uint8_t* smem, const Bars& B, int items,
-                                         uint32_t tmem, int warp, int lane, int rank, int pair,
-                                         int npairs) {
+__device__ __forceinline__ void g1p_weight(const G1Params& P, uint8_t* smem, const Bars& B, int items,
+                                           uint32_t tmem, int warp, int lane, int rank, int pair,
+                                           int npairs) {
   using C = G1PCfg<PREC>;
-  constexpr int STAGES = C::STAGES, SEG = C::SEG, LAG = C::LAG;
   const int lq = warp & 3;
-  const int h = warp >> 2;
-  const int row = lq * 32 + lane;
-  const uint32_t tq = tmem + ((uint32_t)(lq * 32) << 16);
+  const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + G1_ACOL;
   int s = 0;
-  uint32_t ph = 0, aph = 0;
-  bool ok = true;
-  float sum[128];
+  uint32_t ph = 0;
   bool stall = P.stall != 0 && blockIdx.x == 0;
-  for (int item = pair; item < items && ok; item += npairs) {
-    int q, k, I2, J, sp;
-    const TcProblem* pr = g1p_item(P, item, q, k, I2, J, sp);
-    int rb, re;
-    g1_range<C::SUB>(P, pr, q, sp, rb, re);
-    const int ns = pr->ns, ns_pad = pr->ns_pad;
-    const int nseg = (re - rb + SEG - 1) / SEG;
-#pragma unroll
-    for (int c = 0; c < 128; ++c) sum[c] = 0.f;
-    int flushed = 0;
-    for (int rc = rb; rc < re; ++rc) {
-      if (!waitw(&B.full[s], ph, B, P.status)) { ok = false; break; }
-      weight_stage_c<PREC, C>(ptx::smem_u32(smem + s * C::STRIDE), row, h, 1,
-                              tq + (uint32_t)(G1_ACOL + s * C::SLOT));
+  for (int item = pair; item < items; item += npairs) {
+    int n;
+    {
+      G1Item x;
+      const TcProblem* pr = g1p_item(P, item, rank, x);
+      int rb, re;
+      g1_range<C::SUB>(P, pr, x.q, x.split, rb, re);
+      n = re - rb;
+    }
+    for (int i = 0; i < n; ++i) {
+      if (!waitw(&B.full[s], ph, B, P.status)) return;
+      weight_stage_c<PREC, C>(ptx::smem_u32(smem + s * C::STRIDE), lq * 32 + lane, warp >> 2, 1,
+                              ta + (uint32_t)(s * C::SLOT));
       ptx::tmem_wait_st();
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0 && !stall) ptx::mbar_arrive_cluster(&B.ready[s], 0);
       stall = false;
-      if (++s == STAGES) { s = 0; ph ^= 1; }
-      const int ready_seg = (rc - rb + 1 - LAG) / SEG;
-      const bool last = rc + 1 == re;
-      while (flushed < nseg && (flushed < ready_seg || last)) {
-        if (!waitw(&B.acc_full[0], aph, B, P.status)) { ok = false; break; }
-        ptx::tc_fence_after();
-        const uint32_t ta = tq + (uint32_t)(h * 128);
-#pragma unroll
-        for (int c8 = 0; c8 < 8; ++c8) {
-          float v[16];
-          ptx::tmem_ld16(ta + c8 * 16, v);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) sum[c8 * 16 + e] += v[e];
-        }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(&B.acc_empty[0], 0);
-        aph ^= 1;
-        ++flushed;
-      }
-      if (!ok) break;
+      if (++s == C::STAGES) { s = 0; ph ^= 1; }
     }
-    if (!ok) break;
-    const int i = (2 * I2 + rank) * BM + row;
-    if (i < ns) {
-      float* Xk = P.X[q] + ((long long)sp * P.K[q] + k) * ns_pad * ns_pad;
-      const int j0 = J * 256 + h * 128;
+  }
+}
+
+__device__ __forceinline__ void add_cols(uint64_t* sum, const float (&v)[16]) {
 #pragma unroll
-      for (int c = 0; c < 128; ++c) {
-        const int j = j0 + c;
-        if (j >= i && j < ns) {
-          Xk[(long long)i * ns_pad + j] = sum[c];
-          Xk[(long long)j * ns_pad + i] = sum[c];
+  for (int i = 0; i < 8; ++i)
+    sum[i] = ptx::f2_add(sum[i], ptx::f2_pack(__float_as_uint(v[2 * i]), __float_as_uint(v[2 * i + 1])));
+}
+__device__ __forceinline__ float lo_f(uint64_t x) { return __uint_as_float((uint32_t)x); }
+__device__ __forceinline__ float hi_f(uint64_t x) { return __uint_as_float((uint32_t)(x >> 32)); }
+
+// Segment accumulation and the tile's store (warps 8-15 of both CTAs: TMEM lane
+// quarter w % 4, column block (w - 8) / 4).
+template <int PREC>
+__device__ __forceinline__ void g1p_accumulate(const G1Params& P, const Bars& B, int items, uint32_t tmem,
+                                               int warp, int lane, int rank, int pair, int npairs) {
+  using C = G1PCfg<PREC>;
+  const int lq = warp & 3, h = (warp >> 2) & 1;
+  const uint32_t ta = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)(h * 128);
+  uint32_t ph = 0;
+  for (int item = pair; item < items; item += npairs) {
+    int nseg;
+    {
+      G1Item x;
+      const TcProblem* pr = g1p_item(P, item, rank, x);
+      int rb, re;
+      g1_range<C::SUB>(P, pr, x.q, x.split, rb, re);
+      nseg = (re - rb + C::SEG - 1) / C::SEG;
+    }
+    uint64_t sum[64];                   // 128 columns, in packed pairs
+#pragma unroll
+    for (int c = 0; c < 64; ++c) sum[c] = 0;
+    for (int sg = 0; sg < nseg; ++sg, ph ^= 1) {
+      if (!waitw(&B.acc_full[0], ph, B, P.status)) return;
+      ptx::tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        float v[16];
+        ptx::tmem_ld16(ta + c * 16, v);
+        if (c == 7) {                   // all read: the MMAs may overwrite
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive_cluster(&B.acc_empty[0], 0);
+        }
+        add_cols(sum + c * 8, v);
+      }
+    }
+    // Block (b, c) as X[i][j] and as X[j][i]: a thread's columns of its row i in
+    // 16-byte stores, the mirrored entries one column a time, consecutive over
+    // the lanes.  In a diagonal block i <= j only.
+    G1Item x;
+    const TcProblem* pr = g1p_item(P, item, rank, x);
+    const int ns = pr->ns, ns_pad = pr->ns_pad;
+    const int i = x.b * BM + lq * 32 + lane, c = h ? x.c1 : x.c0;
+    if (i < ns && !(h && x.c1 == x.c0) && (x.two || c >= x.b)) {
+      float* Xk = P.X[x.q] + ((long long)x.split * P.K[x.q] + x.k) * ns_pad * ns_pad;
+      const int j0 = c * BM, jmin = c == x.b ? i : 0;
+#pragma unroll
+      for (int u = 0; u < 128; u += 4) {
+        const int j = j0 + u;
+        const float v[4] = {lo_f(sum[u / 2]), hi_f(sum[u / 2]), lo_f(sum[u / 2 + 1]), hi_f(sum[u / 2 + 1])};
+        if (j >= jmin && j + 3 < ns) {
+          *reinterpret_cast<float4*>(Xk + (long long)i * ns_pad + j) =
+              make_float4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) Xk[(long long)(j + e) * ns_pad + i] = v[e];
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (j + e >= jmin && j + e < ns) {
+              Xk[(long long)i * ns_pad + j + e] = v[e];
+              Xk[(long long)(j + e) * ns_pad + i] = v[e];
+            }
         }
       }
     }
@@ -1569,7 +1683,7 @@ __device__ __forceinline__ void g1p_math(const G1Params& P, uint8_t* smem, const
 
 // Launched in clusters of two CTAs (an even number of CTAs, one per SM).
 template <int PREC>
-__global__ void __launch_bounds__(G1_THREADS, 1)
+__global__ void __launch_bounds__(G1P_THREADS, 1)
     k_gemm1_pair(const __grid_constant__ G1Params P) {
   using C = G1PCfg<PREC>;
   constexpr int STAGES = C::STAGES;
@@ -1594,7 +1708,7 @@ __global__ void __launch_bounds__(G1_THREADS, 1)
     ptx::fence_barrier_init();
     ptx::fence_proxy_async_smem();
   }
-  if (warp == 9) {
+  if (warp == 17) {
     ptx::tmem_alloc_pair(B.tmem_slot, 512);
     ptx::tmem_relinquish_pair();
   }
@@ -1603,18 +1717,21 @@ __global__ void __launch_bounds__(G1_THREADS, 1)
   ptx::cluster_sync();          // both CTAs' barriers initialised before any remote arrive
   ptx::tc_fence_after();
   const uint32_t tmem = *B.tmem_slot;
-  if (warp >= 8) {
-    ptx::setmaxnreg_dec<G1_REG_CTRL>();
-    if (warp == 8 && lane == 0) g1p_producer<PREC>(P, smem, B, items, rank, pair, npairs);
-    else if (warp == 9 && lane == 0 && rank == 0) g1p_mma<PREC>(P, smem, B, items, tmem, pair, npairs);
+  if (warp >= 16) {
+    ptx::setmaxnreg_dec<G1P_REG_CTRL>();
+    if (warp == 16 && lane == 0) g1p_producer<PREC>(P, smem, B, items, rank, pair, npairs);
+    else if (warp == 17 && lane == 0 && rank == 0) g1p_mma<PREC>(P, smem, B, items, tmem, pair, npairs);
+  } else if (warp >= 8) {
+    ptx::setmaxnreg_inc<G1P_REG_ACC>();
+    g1p_accumulate<PREC>(P, B, items, tmem, warp, lane, rank, pair, npairs);
   } else {
-    ptx::setmaxnreg_inc<G1_REG_MATH>();
-    g1p_math<PREC>(P, smem, B, items, tmem, warp, lane, rank, pair, npairs);
+    ptx::setmaxnreg_dec<G1P_REG_WEIGHT>();
+    g1p_weight<PREC>(P, smem, B, items, tmem, warp, lane, rank, pair, npairs);
   }
   ptx::tc_fence_before();
   __syncthreads();
   ptx::cluster_sync();          // the even CTA's MMAs into this CTA's memory are complete
-  if (warp == 9) {
+  if (warp == 17) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc_pair(tmem, 512);
   }
@@ -1746,6 +1863,12 @@ bool build_problem(const Channel& c, const SysState& S, int ch, TcProblem& pr) {
   pr.ntiles_w = 0;                          // GEMM1 128 x 256 tiles (I below the end of J)
   for (int j = 0; 256 * j < c.ns_pad; ++j) pr.ntiles_w += 2 * (j + 1) < pr.nI ? 2 * (j + 1) : pr.nI;
   pr.ntiles_p = pr.NJ * (pr.NJ + 1) / 2;    // GEMM1 256 x 256 pair tiles with I <= J
+  pr.ntiles_d = 0;
+  const int nb = (c.ns + BM - 1) / BM;      // block rows with states
+  for (int Q = 0; 4 * Q < nb; ++Q) {
+    const int r = nb - 4 * Q < 4 ? nb - 4 * Q : 4;
+    pr.ntiles_d += 2 * r * Q + g1p_group_items(r);
+  }
   pr.nch = (int)(S.Ng_pad / BK);
   pr.nR = (int)(S.Ng_pad / BM);
   pr.kmax = S.kmax;
@@ -1870,7 +1993,7 @@ cudaError_t pair_attr() {
 
 template <int PREC>
 int pair_clusters() {
-  return cluster_pairs(k_gemm1_pair<PREC>, G1PCfg<PREC>::SMEM, G1_THREADS, PairKernels<PREC>::g1_attr,
+  return cluster_pairs(k_gemm1_pair<PREC>, G1PCfg<PREC>::SMEM, G1P_THREADS, PairKernels<PREC>::g1_attr,
                        PairKernels<PREC>::g1_cache, "projection");
 }
 
@@ -1908,7 +2031,7 @@ cudaError_t gemm1_pair_group(const TcEntry* e, int n, int* status, cudaStream_t 
       P.X[q] = static_cast<float*>(x.X);
       P.nsplit[q] = x.split > 1 ? x.split : 1;
       P.begin[q] = items;
-      items += x.host->ntiles_p * x.K * P.nsplit[q];
+      items += tc_g1p_items(*x.host, x.K) * P.nsplit[q];
       const long long nch = nch_lim > 0 && nch_lim < x.host->nch ? nch_lim : x.host->nch;
       const long long len = nch * 1024 / P.nsplit[q];
       if (len0 >= 0 && len != len0) equal = false;
@@ -1929,7 +2052,7 @@ cudaError_t gemm1_pair_group(const TcEntry* e, int n, int* status, cudaStream_t 
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(2 * pairs, 1, 1);
-    cfg.blockDim = dim3(G1_THREADS, 1, 1);
+    cfg.blockDim = dim3(G1P_THREADS, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = at;
@@ -2155,6 +2278,8 @@ bool tc_supported() {
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
   return major == 10 && minor == 3 && encode_fn() != nullptr;
 }
+
+int tc_g1p_items(const TcProblem& pr, int K) { return pr.ntiles_d * (K / 2) + pr.ntiles_p * (K % 2); }
 
 int tc_pair_units(int prec) {
   return prec == LRDM_BF16X3 ? pair_clusters<LRDM_BF16X3>() : pair_clusters<LRDM_TF32>();

@@ -404,7 +404,7 @@ int choose_split(lrdm_ctx* ctx, int s, int K) {
   const bool wide = ctx->tune.g1_nb == 256;
   const int dpt = wide || pair ? 1 : ctx->tune.g1_dpt;
   const long long items =
-      (long long)(pair ? pr.ntiles_p : wide ? pr.ntiles_w : pr.ntiles) * ((K + dpt - 1) / dpt);
+      pair ? tc_g1p_items(pr, K) : (long long)(wide ? pr.ntiles_w : pr.ntiles) * ((K + dpt - 1) / dpt);
   // work units of the persistent grid: SMs, or CTA pairs for the pair tiles
   const long long sms = pair ? tc_pair_units(ctx->opt.prec) : ctx->sm_count > 0 ? ctx->sm_count : 148;
   return tc_split(items, sms, pr.nch, S.xslots / K);
@@ -570,7 +570,7 @@ lrdm_status autotune(lrdm_ctx* ctx, cudaStream_t st) {
     ctx->tune = start;
     if (c[0] == G1_PAIR) {
       long long items = 0;
-      for (const TcEntry& x : g1) items += (long long)x.host->ntiles_p * x.K * (x.split > 1 ? x.split : 1);
+      for (const TcEntry& x : g1) items += (long long)tc_g1p_items(*x.host, x.K) * (x.split > 1 ? x.split : 1);
       if (items < units) continue;
     }
     const float ms = time_launch([&] { return launch_gemm1_tc_group(ctx->opt.prec, g1.data(), (int)g1.size(),

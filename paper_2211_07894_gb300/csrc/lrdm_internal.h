@@ -404,5 +404,6 @@ bool tc_supported();
 // CTA pairs the pair-tile projection kernel keeps resident on the current
 // device (its persistent grid is twice this many CTAs).
 int tc_pair_units(int prec);
+int tc_g1p_items(const TcProblem& pr, int K);   // work items of the pair projection of K directions
 
 }  // namespace lrdm

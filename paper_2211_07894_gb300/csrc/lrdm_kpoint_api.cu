@@ -70,7 +70,7 @@ int kp_choose_split(lrdm_ctx* ctx, int K) {
     const TcProblem& pr = ctx->tc_host[ctx->kp_pid[q]];
     const bool wide = ctx->tune.g1_nb == 256;
     const int dpt = wide || pair ? 1 : ctx->tune.g1_dpt;
-    per += (long long)(pair ? pr.ntiles_p : wide ? pr.ntiles_w : pr.ntiles) * ((K + dpt - 1) / dpt);
+    per += pair ? tc_g1p_items(pr, K) : (long long)(wide ? pr.ntiles_w : pr.ntiles) * ((K + dpt - 1) / dpt);
     nch = std::min(nch, pr.nch);
   }
   return tc_split(per, sms, nch, ctx->kp_split_cap);

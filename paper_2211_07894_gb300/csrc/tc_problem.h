@@ -20,7 +20,8 @@ struct TcProblem {
   const void* psi1;                      // bf16 lo
   double* part;                          // GEMM2 j-tile part sums [G2_MAX_SPLIT][Ng] (small K)
   int ns, ns_pad, nI, NJ, ntiles, ntiles_w, nch, nR, kmax;   // GEMM1: nI blocks, ntiles tiles; GEMM2: NJ, nR
-  int ntiles_p;                          // GEMM1 on CTA pairs: 256 x 256 tiles with I <= J
+  int ntiles_p;                          // GEMM1 on CTA pairs: 256 x 256 tiles with I <= J (one direction)
+  int ntiles_d;                          // ... and items of one row block, two column blocks, two directions
 };
 
 constexpr int TC_MAX_SLOTS = 16;        // problems per grouped launch
