@@ -33,6 +33,18 @@ __device__ __forceinline__ double block_sum(double x, double* sh) {
   return s;                             // valid in thread 0
 }
 
+// Sum of n partials `stride` apart, by one warp (in all lanes): every block of
+// k_gs_axpy and k_normalize adds up the same KR_BLOCKS partials.  One thread
+// doing it was a chain of 304 loads and adds: 48^3, K = 4: k_gs_axpy 20-24 ->
+// 8-10 us, k_normalize 20 -> 6.5 us (64^3: the same).
+__device__ __forceinline__ double warp_sum(const double* __restrict__ p, long long stride, int n) {
+  double s = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x & 31; b < n; b += 32) s += p[b * stride];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
 // partial[b][k] = sum over this block's points of t u_k
 __global__ void __launch_bounds__(KR_THREADS) k_dots(const void* __restrict__ U, int K,
                                                      const void* __restrict__ t, int io, long long n,
@@ -57,16 +69,16 @@ __global__ void __launch_bounds__(KR_THREADS) k_gs_axpy(const void* __restrict__
                                                         double* __restrict__ npart) {
   __shared__ double c[KMAX_LIMIT];
   __shared__ double sh[32];
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partial[(long long)b * K + k];
-    c[k] = w * s;
+  for (int k = threadIdx.x >> 5; k < K; k += blockDim.x >> 5) {
+    const double s = warp_sum(partial + k, K, nblk);
+    if ((threadIdx.x & 31) == 0) c[k] = w * s;
   }
   __syncthreads();
   double acc = 0.0;
   for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n;
        r += (long long)gridDim.x * blockDim.x) {
     double x = ld_io(t, io, r);
+#pragma unroll 4
     for (int k = 0; k < K; ++k) x -= c[k] * ld_io(U, io, (long long)k * n + r);
     st_io(out, io, r, x);
     acc += x * x;
@@ -80,11 +92,12 @@ __global__ void __launch_bounds__(KR_THREADS) k_normalize(void* __restrict__ out
                                                           double w, const double* __restrict__ npart,
                                                           int nblk, double* __restrict__ norm_out) {
   __shared__ double nrm;
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += npart[b];
-    nrm = sqrt(w * s);
-    if (blockIdx.x == 0 && norm_out) norm_out[0] = nrm;
+  if (threadIdx.x < 32) {
+    const double s = warp_sum(npart, 1, nblk);
+    if (threadIdx.x == 0) {
+      nrm = sqrt(w * s);
+      if (blockIdx.x == 0 && norm_out) norm_out[0] = nrm;
+    }
   }
   __syncthreads();
   if (!(nrm > 0.0)) return;
