@@ -8,8 +8,11 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <cudaTypedefs.h>
+
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -112,6 +115,121 @@ lrdm_status validate_system(const lrdm_system& s, const lrdm_options& o) {
   return LRDM_OK;
 }
 
+// cuFFT plans of closed contexts, for the next context of the same transform: a
+// pair of plans takes 0.7 ms to make and 0.07 ms to destroy, and a
+// self-consistency loop makes a context a step (48^3, N_s = 512: create 1.65 ->
+// 0.99 ms, destroy 0.91 -> 0.82 ms).  A pair belongs to one context from take()
+// to give(), which its context calls after a device synchronisation.  At most
+// POOL_PAIRS pairs and POOL_BYTES of their work areas wait here; the oldest go
+// first, and all of them when an allocation fails.  The key holds the CUDA
+// context's id, so that none is used in another one or after a reset.
+class PlanPool {
+ public:
+  PlanPool() { idle_.reserve(POOL_PAIRS + 1); }
+  struct Key {
+    unsigned long long ctx = 0;
+    int n[3] = {0, 0, 0}, batch = 0, fp64 = 0;
+    bool operator==(const Key& o) const {
+      return ctx == o.ctx && n[0] == o.n[0] && n[1] == o.n[1] && n[2] == o.n[2] && batch == o.batch && fp64 == o.fp64;
+    }
+  };
+  // The id of the current CUDA context, 0 if it cannot be told (nothing is kept then).
+  static unsigned long long context_id() {
+    static const PFN_cuCtxGetId_v12000 fn = [] {
+      void* p = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+          q == cudaDriverEntryPointSuccess)
+        return reinterpret_cast<PFN_cuCtxGetId_v12000>(p);
+      return (PFN_cuCtxGetId_v12000) nullptr;
+    }();
+    unsigned long long id = 0;
+    return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+  }
+  bool take(const Key& k, cufftHandle* r2c, cufftHandle* c2r) {
+    std::lock_guard<std::mutex> g(m_);
+    for (size_t i = idle_.size(); k.ctx && i-- > 0;)
+      if (idle_[i].key == k) {
+        *r2c = idle_[i].r2c;
+        *c2r = idle_[i].c2r;
+        idle_.erase(idle_.begin() + (long)i);
+        return true;
+      }
+    return false;
+  }
+  void give(const Key& k, cufftHandle r2c, cufftHandle c2r) {
+    size_t a = 0, b = 0;
+    if (!k.ctx || k.ctx != context_id() || cufftGetSize(r2c, &a) != CUFFT_SUCCESS ||
+        cufftGetSize(c2r, &b) != CUFFT_SUCCESS || a + b > POOL_BYTES) {
+      cufftDestroy(r2c);
+      cufftDestroy(c2r);
+      return;
+    }
+    std::lock_guard<std::mutex> g(m_);
+    idle_.push_back(Pair{k, r2c, c2r, a + b});
+    size_t sum = 0;
+    for (const Pair& x : idle_) sum += x.bytes;
+    while (idle_.size() > POOL_PAIRS || sum > POOL_BYTES) {
+      sum -= idle_.front().bytes;
+      drop_front(k.ctx);
+    }
+  }
+  // Destroys what waits; whether anything did.
+  bool clear() {
+    const unsigned long long id = context_id();
+    std::lock_guard<std::mutex> g(m_);
+    const bool any = !idle_.empty();
+    while (!idle_.empty()) drop_front(id);
+    return any;
+  }
+
+ private:
+  static constexpr size_t POOL_PAIRS = 4, POOL_BYTES = 32u << 20;
+  struct Pair {
+    Key key;
+    cufftHandle r2c, c2r;
+    size_t bytes;
+  };
+  void drop_front(unsigned long long current) {
+    if (idle_.front().key.ctx == current) {     // (another context's plans end with it)
+      cufftDestroy(idle_.front().r2c);
+      cufftDestroy(idle_.front().c2r);
+    }
+    idle_.erase(idle_.begin());
+  }
+  std::mutex m_;
+  std::vector<Pair> idle_;
+};
+
+// never destroyed: the CUDA runtime may end before static objects do
+PlanPool& plan_pool() {
+  static PlanPool* pool = new PlanPool;
+  return *pool;
+}
+bool release_idle() { return plan_pool().clear(); }
+
+PlanPool::Key plan_key(const SysState& S) {
+  PlanPool::Key k;
+  k.ctx = S.plan_ctx;
+  for (int d = 0; d < 3; ++d) k.n[d] = S.n[d];
+  k.batch = S.kmax;
+  k.fp64 = S.plan_fp64;
+  return k;
+}
+
+lrdm_status make_plans(SysState& S, int fp64, long long nc) {
+  int nn[3] = {S.n[0], S.n[1], S.n[2]};
+  LRDM_FFT(cufftPlanMany(&S.plan_r2c, 3, nn, nullptr, 1, (int)S.Ngrid, nullptr, 1, (int)nc,
+                         fp64 ? CUFFT_D2Z : CUFFT_R2C, S.kmax));
+  const cufftResult r = cufftPlanMany(&S.plan_c2r, 3, nn, nullptr, 1, (int)nc, nullptr, 1, (int)S.Ngrid,
+                                      fp64 ? CUFFT_Z2D : CUFFT_C2R, S.kmax);
+  if (r != CUFFT_SUCCESS) {
+    cufftDestroy(S.plan_r2c);
+    S.plan_r2c = 0;
+  }
+  return from_cufft(r);
+}
+
 // Poisson: batched real <-> half-complex transforms over k_max fields, the
 // symbol table and the transform buffers of system S.
 lrdm_status setup_poisson(lrdm_ctx* ctx, SysState& S, cudaStream_t st) {
@@ -121,12 +239,14 @@ lrdm_status setup_poisson(lrdm_ctx* ctx, SysState& S, cudaStream_t st) {
   const long long nc = (long long)S.n[0] * S.n[1] * (S.n[2] / 2 + 1);
   LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&S.fft_real), (size_t)S.kmax * S.Ngrid * csz));
   LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&S.fft_cplx), (size_t)S.kmax * nc * 2 * csz));
-  int nn[3] = {S.n[0], S.n[1], S.n[2]};
-  LRDM_FFT(cufftPlanMany(&S.plan_r2c, 3, nn, nullptr, 1, (int)S.Ngrid, nullptr, 1, (int)nc,
-                         fp64 ? CUFFT_D2Z : CUFFT_R2C, S.kmax));
+  S.plan_fp64 = fp64;
+  S.plan_ctx = PlanPool::context_id();
+  if (!plan_pool().take(plan_key(S), &S.plan_r2c, &S.plan_c2r)) {
+    lrdm_status rc = make_plans(S, fp64, nc);
+    if (rc == LRDM_ERR_OOM && release_idle()) rc = make_plans(S, fp64, nc);
+    LRDM_CK(rc);
+  }
   S.plans = true;
-  LRDM_FFT(cufftPlanMany(&S.plan_c2r, 3, nn, nullptr, 1, (int)nc, nullptr, 1, (int)S.Ngrid,
-                         fp64 ? CUFFT_Z2D : CUFFT_C2R, S.kmax));
   LRDM_CK(dalloc(ctx, &S.sym, (size_t)nc, false));
   LRDM_CU(launch_poisson_table(S.n, S.h, o.poisson_symbol, S.sym, st));
   return LRDM_OK;
@@ -743,8 +863,7 @@ void free_ctx(lrdm_ctx* ctx) {
   cudaDeviceSynchronize();
   for (int s = 0; s < ctx->nsys; ++s) {
     SysState& S = ctx->sys[s];
-    if (S.plan_r2c) cufftDestroy(S.plan_r2c);
-    if (S.plan_c2r) cufftDestroy(S.plan_c2r);
+    if (S.plans) plan_pool().give(plan_key(S), S.plan_r2c, S.plan_c2r);
   }
   if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
   for (cudaEvent_t e : ctx->prof_ev) cudaEventDestroy(e);

@@ -155,6 +155,8 @@ struct SysState {
   // Poisson
   cufftHandle plan_r2c = 0, plan_c2r = 0;
   bool plans = false;
+  int plan_fp64 = 0;                 // their precision and the id of the CUDA context they were made in
+  unsigned long long plan_ctx = 0;
   void* fft_real = nullptr;          // [kmax][Ngrid] compute type
   void* fft_cplx = nullptr;          // [kmax][n0][n1][n2/2+1]
   double* sym = nullptr;             // [n0][n1][n2/2+1] Poisson symbol / N_g
@@ -187,6 +189,8 @@ struct lrdm_ctx {
   double* gs_scratch = nullptr;      // Gram-Schmidt partial sums (Krylov step)
   double* gs_norm = nullptr;         // [1] norm of the last normalised direction
   std::vector<void*> allocs;         // every device allocation, freed by lrdm_destroy
+  char* arena = nullptr;             // rest of the last block of small buffers (dalloc)
+  size_t arena_left = 0;
   // tensor-core problem table: one entry per (system, channel)
   std::vector<lrdm::TcProblem> tc_host;
   lrdm::TcProblem* tc_dev = nullptr;
