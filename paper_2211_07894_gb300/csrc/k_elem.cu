@@ -419,11 +419,17 @@ __global__ void k_trace_bar(DmuArgs A, int acc64, double* __restrict__ tbar) {
   if (threadIdx.x == 0) tbar[blockIdx.x] = num;
 }
 
-// One block per state i of channel s:
+// One block of 256 threads per state i of channel s:
 //   Lbar_ij = sum_k G_k,ij (X_k,ij - delta_ij mu'_k) - delta_ij sum_k tbar_k/s (X_k,ii - mu'_k)
 //   eps_bar_i = sum_{j != i, |de| > tau} 2 Lbar_ij (-L_ij / (eps_i - eps_j))
 //   occ_bar_i = sum_{j != i, |de| > tau} 2 Lbar_ij / (eps_i - eps_j)
 //             + sum_{j != i, |de| <= tau} 2 Lbar_ij (-(1 - 2 fbar)/(2 kT)) + Lbar_ii (-(1 - 2 f_i)/kT)
+//
+// Bound by the latency of its loads (K nsplit of X and of G an entry, from L2),
+// so the directions of a row are shared out where threads are left over, and
+// the diagonal's FP64 sums are one direction a lane: 48^3, N_s = 512, K = 8,
+// seven row ranges: 116 -> 32 us (one thread summed the diagonal, 56 terms one
+// after the other).  Four blocks an SM: with two the FP32 form took 41 us.
 //
 // With FP32 partials (the tensor-core and FP32 modes) Lbar_ij (j != i) is
 // summed over the directions in FP32, four consecutive j per thread with
@@ -459,58 +465,79 @@ __device__ __forceinline__ void eob_term(const EobArgs& a, int i, int j, double 
   }
 }
 
-// Lbar_ij in FP64 (the FP64 mode, and the diagonal in every mode)
+// Four columns from j0 of row i, without the diagonal.
+__device__ __forceinline__ void eob_quad(const EobArgs& a, int i, int j0, double eps_i, const float (&acc)[4],
+                                         int ns, double& eb, double& ob, float& ebf, float& obf) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    if (j0 + e < ns && j0 + e != i) eob_term(a, i, j0 + e, eps_i, (double)acc[e], ns, eb, ob, ebf, obf);
+}
+
+// Direction k's part of Lbar_ij in FP64 (the FP64 mode, and the diagonal in
+// every mode).
+__device__ __forceinline__ double eob_lbar64_k(const void* X, const void* G, int acc64, int nsplit,
+                                               int K, int k, long long mat, long long row, int i, int j,
+                                               const double* dmu, const double* tbar,
+                                               double inv_trace) {
+  double x = 0.0, gg = 0.0;
+  for (int p = 0; p < nsplit; ++p) {
+    const long long o = ((long long)p * K + k) * mat + row + j;
+    x += ld_c(X, acc64, o);
+    gg += ld_c(G, acc64, o);
+  }
+  return i == j ? gg * (x - dmu[k]) - tbar[k] * inv_trace * (x - dmu[k]) : gg * x;
+}
 __device__ __forceinline__ double eob_lbar64(const void* X, const void* G, int acc64, int nsplit,
                                              int K, long long mat, long long row, int i, int j,
                                              const double* dmu, const double* tbar,
                                              double inv_trace) {
   double lb = 0.0;
-  for (int k = 0; k < K; ++k) {
-    double x = 0.0, gg = 0.0;
-    for (int p = 0; p < nsplit; ++p) {
-      const long long o = ((long long)p * K + k) * mat + row + j;
-      x += ld_c(X, acc64, o);
-      gg += ld_c(G, acc64, o);
-    }
-    if (i == j) lb += gg * (x - dmu[k]) - tbar[k] * inv_trace * (x - dmu[k]);
-    else lb += gg * x;
-  }
+  for (int k = 0; k < K; ++k) lb += eob_lbar64_k(X, G, acc64, nsplit, K, k, mat, row, i, j, dmu, tbar, inv_trace);
   return lb;
 }
 
-__global__ void k_eps_occ_bar(const void* __restrict__ X, const void* __restrict__ G, int acc64,
-                              int nsplit, int K, int ns, int ldx, EobArgs a,
-                              const double* __restrict__ dmu, const double* __restrict__ tbar,
-                              double inv_trace, double* __restrict__ eps_bar,
-                              double* __restrict__ occ_bar) {
+template <bool ACC64>
+__global__ void __launch_bounds__(256, ACC64 ? 2 : 4)
+    k_eps_occ_bar(const void* __restrict__ X, const void* __restrict__ G, int nsplit, int K, int ns, int ldx,
+                  EobArgs a, const double* __restrict__ dmu, const double* __restrict__ tbar, double inv_trace,
+                  double* __restrict__ eps_bar, double* __restrict__ occ_bar) {
   const int i = blockIdx.x;
   const long long mat = (long long)ldx * ldx;
   const long long row = (long long)i * ldx;
   double eb = 0.0, ob = 0.0;
   float ebf = 0.f, obf = 0.f;
   const double eps_i = a.eps[i];
-  if (!acc64 && ldx % 4 == 0) {
+  constexpr int acc64 = ACC64;
+  if (!ACC64 && ldx % 4 == 0) {
     // FP32 partials: rows of 16-byte quads (ldx is a multiple of 4, so a quad
-    // starting below ns stays inside the padded row)
+    // starting below ns stays inside the padded row).  A row of fewer quads than
+    // threads is taken by several groups of them, each with every G-th
+    // direction, added up in order by the first.
     const float* Xf = static_cast<const float*>(X);
     const float* Gf = static_cast<const float*>(G);
-    for (int j0 = 4 * threadIdx.x; j0 < ns; j0 += 4 * blockDim.x) {
+    const int quads = (ns + 3) / 4;
+    const int ng = min(K, max(1, (int)blockDim.x / quads));
+    const int grp = ng > 1 ? threadIdx.x / quads : 0;
+    const int j00 = 4 * (ng > 1 ? threadIdx.x - grp * quads : threadIdx.x);
+    __shared__ float4 part[256];
+    for (int j0 = j00; j0 < ns && grp < ng; j0 += ng > 1 ? ns : 4 * blockDim.x) {
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      auto add = [&](const float4& g, const float4& x) {
+        acc[0] = fmaf(g.x, x.x, acc[0]);
+        acc[1] = fmaf(g.y, x.y, acc[1]);
+        acc[2] = fmaf(g.z, x.z, acc[2]);
+        acc[3] = fmaf(g.w, x.w, acc[3]);
+      };
       if (nsplit == 1) {
-        // one partial: unrolled so that several directions' loads are in flight
 #pragma unroll 4
-        for (int k = 0; k < K; ++k) {
+        for (int k = grp; k < K; k += ng) {
           const long long o = (long long)k * mat + row + j0;
-          const float4 x = *reinterpret_cast<const float4*>(Xf + o);
-          const float4 g = *reinterpret_cast<const float4*>(Gf + o);
-          acc[0] = fmaf(g.x, x.x, acc[0]);
-          acc[1] = fmaf(g.y, x.y, acc[1]);
-          acc[2] = fmaf(g.z, x.z, acc[2]);
-          acc[3] = fmaf(g.w, x.w, acc[3]);
+          add(*reinterpret_cast<const float4*>(Gf + o), *reinterpret_cast<const float4*>(Xf + o));
         }
       } else {
-        for (int k = 0; k < K; ++k) {
+        for (int k = grp; k < K; k += ng) {
           float4 x = make_float4(0.f, 0.f, 0.f, 0.f), g = x;
+#pragma unroll 4
           for (int p = 0; p < nsplit; ++p) {
             const long long o = ((long long)p * K + k) * mat + row + j0;
             const float4 xv = *reinterpret_cast<const float4*>(Xf + o);
@@ -518,20 +545,31 @@ __global__ void k_eps_occ_bar(const void* __restrict__ X, const void* __restrict
             x.x += xv.x; x.y += xv.y; x.z += xv.z; x.w += xv.w;
             g.x += gv.x; g.y += gv.y; g.z += gv.z; g.w += gv.w;
           }
-          acc[0] = fmaf(g.x, x.x, acc[0]);
-          acc[1] = fmaf(g.y, x.y, acc[1]);
-          acc[2] = fmaf(g.z, x.z, acc[2]);
-          acc[3] = fmaf(g.w, x.w, acc[3]);
+          add(g, x);
         }
       }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int j = j0 + e;
-        if (j >= ns) break;
-        const double lb = j == i ? eob_lbar64(X, G, 0, nsplit, K, mat, row, i, j, dmu, tbar, inv_trace)
-                                 : (double)acc[e];
-        eob_term(a, i, j, eps_i, lb, ns, eb, ob, ebf, obf);
+      if (ng > 1) part[threadIdx.x] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      else eob_quad(a, i, j0, eps_i, acc, ns, eb, ob, ebf, obf);
+    }
+    if (ng > 1) {
+      __syncthreads();
+      if (threadIdx.x < quads) {
+        float4 v = part[threadIdx.x];
+        for (int g = 1; g < ng; ++g) {
+          const float4 u = part[g * quads + threadIdx.x];
+          v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+        }
+        const float acc[4] = {v.x, v.y, v.z, v.w};
+        eob_quad(a, i, j00, eps_i, acc, ns, eb, ob, ebf, obf);
       }
+    }
+    // the diagonal in FP64: the last warp, a direction a lane
+    if ((int)threadIdx.x >= (int)blockDim.x - 32) {
+      double lb = 0.0;
+      for (int k = threadIdx.x & 31; k < K; k += 32)
+        lb += eob_lbar64_k(X, G, 0, nsplit, K, k, mat, row, i, i, dmu, tbar, inv_trace);
+      for (int o = 16; o > 0; o >>= 1) lb += __shfl_xor_sync(0xffffffffu, lb, o);
+      if ((threadIdx.x & 31) == 0) eob_term(a, i, i, eps_i, lb, ns, eb, ob, ebf, obf);
     }
   } else {
     for (int j = threadIdx.x; j < ns; j += blockDim.x) {
@@ -759,7 +797,11 @@ cudaError_t launch_eps_occ_bar(const SysState& S, int s, int K, int acc_fp64, do
   int ldx = tc ? c.ns_pad : c.ns;
   // the FP32 copy of L exists in the tensor-core modes (leading dimension ns_pad)
   EobArgs a{c.L, acc_fp64 ? nullptr : c.Lf, c.ns_pad, c.eps, c.occ, S.kT, degen_tol * S.kT};
-  k_eps_occ_bar<<<c.ns, 256, 0, st>>>(c.Xpart, c.Gpart, acc_fp64, S.nsplit, K, c.ns, ldx, a, S.dmu,
+  if (acc_fp64)
+    k_eps_occ_bar<true><<<c.ns, 256, 0, st>>>(c.Xpart, c.Gpart, S.nsplit, K, c.ns, ldx, a, S.dmu,
+                                      S.tbar, inv_trace_L, eps_bar, occ_bar);
+  else
+    k_eps_occ_bar<false><<<c.ns, 256, 0, st>>>(c.Xpart, c.Gpart, S.nsplit, K, c.ns, ldx, a, S.dmu,
                                       S.tbar, inv_trace_L, eps_bar, occ_bar);
   return cudaGetLastError();
 }
