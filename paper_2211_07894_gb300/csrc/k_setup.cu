@@ -33,53 +33,85 @@ __global__ void k_copy_rowmajor(const void* __restrict__ src, int io_dtype, int 
   }
 }
 
-// Padded row-major [Ng_pad][ns_pad] and transposed (tile-major, see below)
-// copies for the tensor-core paths; split into bf16 hi/lo (x = hi + lo,
-// lo = bf16(x - hi)) or rounded to TF32.  Tiled transpose through shared memory.
-__global__ void k_copy_tc(const void* __restrict__ src, int io_dtype, int ld, long long Ng, int ns,
-                          long long Ng_pad, int ns_pad, float* __restrict__ R32,
-                          float* __restrict__ T32, __nv_bfloat16* __restrict__ Rhi,
-                          __nv_bfloat16* __restrict__ Rlo, __nv_bfloat16* __restrict__ Thi,
-                          __nv_bfloat16* __restrict__ Tlo, float* __restrict__ Tf) {
-  __shared__ float tile[32][33];
-  long long r0 = (long long)blockIdx.x * 32;
-  int i0 = blockIdx.y * 32;
-  int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  for (int yy = ty; yy < 32; yy += 8) {
-    long long r = r0 + yy;
-    int i = i0 + tx;
-    float x = 0.f;
-    if (r < Ng && i < ns) x = (float)load_io(src, io_dtype, r * ld + i);
-    tile[yy][tx] = x;
-    if (r < Ng_pad && i < ns_pad) {
-      long long o = r * ns_pad + i;
-      if (R32) R32[o] = to_tf32(x);
-      if (Rhi) {
-        __nv_bfloat16 hi = __float2bfloat16_rn(x);
-        Rhi[o] = hi;
-        Rlo[o] = __float2bfloat16_rn(x - __bfloat162float(hi));
+__device__ __forceinline__ uint32_t pack_bf2(__nv_bfloat16 a, __nv_bfloat16 b) {
+  const __nv_bfloat162 v = __halves2bfloat162(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// x = hi + lo: four values as 8 bytes of hi and of lo
+__device__ __forceinline__ void split4(const float (&x)[4], uint2& hi, uint2& lo) {
+  __nv_bfloat16 h[4], l[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    h[c] = __float2bfloat16_rn(x[c]);
+    l[c] = __float2bfloat16_rn(x[c] - __bfloat162float(h[c]));
+  }
+  hi = make_uint2(pack_bf2(h[0], h[1]), pack_bf2(h[2], h[3]));
+  lo = make_uint2(pack_bf2(l[0], l[1]), pack_bf2(l[2], l[3]));
+}
+
+// Padded row-major [Ng_pad][ns_pad] and transposed tile-major copies for the
+// tensor-core paths; split into bf16 hi/lo (x = hi + lo, lo = bf16(x - hi)) or
+// rounded to TF32.  The transposed copies are [i / 128][r / RB][i % 128][r % RB]
+// with RB = 64 bytes of the operand type (16 TF32, 32 bf16; the exact FP32 copy
+// of the split mode shares the bf16 RB = 32), so that one (128 states x RB rows)
+// tensor-core operand tile is a contiguous block.
+//
+// A block converts 32 rows x 128 states through shared memory: one such tile of
+// the split mode (8 or 16 KB written in a piece), two of TF32.  Bound by HBM
+// (20 bytes a value split, 12 TF32); four values a thread, 16-byte loads (vec:
+// FP32 rows on 16-byte boundaries) and 8- or 16-byte stores.  48^3, N_s = 512:
+// 239 -> 133 us (32 x 32 tiles with 2-byte stores before; 135 us at the copy
+// rate).
+__global__ void __launch_bounds__(256)
+    k_copy_tc(const void* __restrict__ src, int io_dtype, int ld, long long Ng, int ns, long long Ng_pad,
+              int ns_pad, int vec, float* __restrict__ R32, float* __restrict__ T32,
+              __nv_bfloat16* __restrict__ Rhi, __nv_bfloat16* __restrict__ Rlo,
+              __nv_bfloat16* __restrict__ Thi, __nv_bfloat16* __restrict__ Tlo, float* __restrict__ Tf) {
+  __shared__ float tile[128][33];                  // [state][row]
+  const long long r0 = (long long)blockIdx.x * 32;
+  const int i0 = blockIdx.y * 128;
+  for (int e = threadIdx.x; e < 32 * 32; e += 256) {
+    const int rr = e >> 5, ii = 4 * (e & 31), i = i0 + ii;
+    const long long r = r0 + rr;
+    float x[4] = {0.f, 0.f, 0.f, 0.f};
+    if (r < Ng) {
+      if (vec && i + 3 < ns) {
+        const float4 v = *reinterpret_cast<const float4*>(static_cast<const float*>(src) + r * ld + i);
+        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (i + c < ns) x[c] = (float)load_io(src, io_dtype, r * ld + i + c);
       }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) tile[ii + c][rr] = x[c];
+    const long long o = r * ns_pad + i;            // (Ng_pad and ns_pad are multiples of 128)
+    if (R32) *reinterpret_cast<float4*>(R32 + o) =
+        make_float4(to_tf32(x[0]), to_tf32(x[1]), to_tf32(x[2]), to_tf32(x[3]));
+    if (Rhi) {
+      uint2 hi, lo;
+      split4(x, hi, lo);
+      *reinterpret_cast<uint2*>(Rhi + o) = hi;
+      *reinterpret_cast<uint2*>(Rlo + o) = lo;
     }
   }
   __syncthreads();
-  // transposed copies are tile-major: [i / 128][r / RB][i % 128][r % RB] with
-  // RB = 64 bytes of the operand type (16 TF32, 32 bf16; the exact FP32 copy
-  // of the split mode shares the bf16 RB = 32), so that one (128 states x RB
-  // rows) tensor-core operand tile is a contiguous block
-  for (int yy = ty; yy < 32; yy += 8) {
-    int i = i0 + yy;
-    long long r = r0 + tx;
-    if (i < ns_pad && r < Ng_pad) {
-      float x = tile[tx][yy];
-      const int RB = T32 ? 16 : 32;
-      long long o = (((long long)(i >> 7) * (Ng_pad / RB) + r / RB) * 128 + (i & 127)) * RB + r % RB;
-      if (T32) T32[o] = to_tf32(x);
+  for (int e = threadIdx.x; e < 128 * 8; e += 256) {
+    const int ii = e >> 3, rr = 4 * (e & 7);
+    const float x[4] = {tile[ii][rr], tile[ii][rr + 1], tile[ii][rr + 2], tile[ii][rr + 3]};
+    if (T32) {
+      const long long o = (((long long)blockIdx.y * (Ng_pad / 16) + (r0 + rr) / 16) * 128 + ii) * 16 + rr % 16;
+      *reinterpret_cast<float4*>(T32 + o) = make_float4(to_tf32(x[0]), to_tf32(x[1]), to_tf32(x[2]), to_tf32(x[3]));
+    } else {
+      const long long o = (((long long)blockIdx.y * (Ng_pad / 32) + blockIdx.x) * 128 + ii) * 32 + rr;
       if (Thi) {
-        __nv_bfloat16 hi = __float2bfloat16_rn(x);
-        Thi[o] = hi;
-        Tlo[o] = __float2bfloat16_rn(x - __bfloat162float(hi));
+        uint2 hi, lo;
+        split4(x, hi, lo);
+        *reinterpret_cast<uint2*>(Thi + o) = hi;
+        *reinterpret_cast<uint2*>(Tlo + o) = lo;
       }
-      if (Tf) Tf[o] = x;
+      if (Tf) *reinterpret_cast<float4*>(Tf + o) = make_float4(x[0], x[1], x[2], x[3]);
     }
   }
 }
@@ -182,13 +214,26 @@ __device__ double loewner_T(double ei, double ej, double mu, double kT, int T) {
   return -exp(lm);
 }
 
-__global__ void k_loewner(const double* __restrict__ eps, const double* __restrict__ occ, int ns,
-                          double mu, double kT, int occ_mode, double degen_tol, int fermi_T,
-                          double* __restrict__ L) {
-  long long total = (long long)ns * ns;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    int i = (int)(e / ns), j = (int)(e - (long long)i * ns);
+// A block takes the 32 x 32 entries (I, J), I <= J, and writes them to (J, I) as
+// well: L is symmetric.  cosh(x / 2) of its 64 states once, a sinh and two
+// divisions an entry remain; FP64-bound.  N_s = 512: 64 -> 22 us.
+__global__ void __launch_bounds__(256)
+    k_loewner(const double* __restrict__ eps, const double* __restrict__ occ, int ns, double mu, double kT,
+              int occ_mode, double degen_tol, int fermi_T, double* __restrict__ L) {
+  __shared__ double xs[64], ch[64];                // x = (eps - mu) / kT and cosh(x / 2) of rows, columns
+  int I = 0, t = blockIdx.x;                       // block t: column J = I + t of row I of the triangle
+  for (int len = (ns + 31) / 32; t >= len; --len, ++I) t -= len;
+  const int i0 = 32 * I, j0 = 32 * (I + t);
+  if (threadIdx.x < 64) {
+    const int q = threadIdx.x < 32 ? i0 + threadIdx.x : j0 + threadIdx.x - 32;
+    const double x = q < ns ? (eps[q] - mu) / kT : 0.0;
+    xs[threadIdx.x] = x;
+    ch[threadIdx.x] = cosh(0.5 * x);
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < 1024; e += 256) {
+    const int li = e >> 5, lj = e & 31, i = i0 + li, j = j0 + lj;
+    if (j < i || j >= ns) continue;
     double val;
     if (fermi_T > 0) {
       val = loewner_T(eps[i], eps[j], mu, kT, fermi_T);
@@ -201,17 +246,18 @@ __global__ void k_loewner(const double* __restrict__ eps, const double* __restri
         val = (occ[i] - occ[j]) / de;
       }
     } else {
-      double xi = (eps[i] - mu) / kT, xj = (eps[j] - mu) / kT;
+      double xi = xs[li], xj = xs[32 + lj];
       double u = 0.5 * (xi - xj);
       if (fabs(xi) < 700.0 && fabs(xj) < 700.0 && fabs(u) < 700.0) {
         double sc = (u == 0.0) ? 1.0 : sinh(u) / u;
-        val = -sc / (4.0 * kT * cosh(0.5 * xi) * cosh(0.5 * xj));
+        val = -sc / (4.0 * kT * ch[li] * ch[32 + lj]);
       } else {
         double lm = log_sinhc(u) - log(4.0 * kT) - log_cosh(0.5 * xi) - log_cosh(0.5 * xj);
         val = -exp(lm);
       }
     }
-    L[e] = val;
+    L[(long long)i * ns + j] = val;
+    L[(long long)j * ns + i] = val;
   }
 }
 
@@ -240,10 +286,11 @@ cudaError_t launch_convert_psi(const void* src, int io_dtype, int ld, long long 
                                                              c.psi32);
     return cudaGetLastError();
   }
-  dim3 blk(32, 8);
-  dim3 grd((unsigned)((Ng_pad + 31) / 32), (unsigned)((c.ns_pad + 31) / 32));
-  k_copy_tc<<<grd, blk, 0, st>>>(src, io_dtype, ld, Ng, ns, Ng_pad, c.ns_pad, c.psiR32, c.psiT32,
-                                 c.psiR_hi, c.psiR_lo, c.psiT_hi, c.psiT_lo, c.psiTf);
+  static_assert(TC_PAD_GRID % 32 == 0 && TC_PAD_STATES == 128, "tiles of k_copy_tc");
+  const int vec = io_dtype == LRDM_DTYPE_F32 && ld % 4 == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+  k_copy_tc<<<dim3((unsigned)(Ng_pad / 32), (unsigned)(c.ns_pad / 128)), 256, 0, st>>>(
+      src, io_dtype, ld, Ng, ns, Ng_pad, c.ns_pad, vec, c.psiR32, c.psiT32, c.psiR_hi, c.psiR_lo, c.psiT_hi,
+      c.psiT_lo, c.psiTf);
   return cudaGetLastError();
 }
 
@@ -270,8 +317,8 @@ cudaError_t launch_fx(const double* rho, long long Ng, int spin_polarized, doubl
 cudaError_t launch_loewner(const double* eps, const double* occ, int ns, double mu, double kT,
                            int occ_mode, double degen_tol, int fermi_T, double* L,
                            cudaStream_t st) {
-  k_loewner<<<grid_for((long long)ns * ns, 256), 256, 0, st>>>(eps, occ, ns, mu, kT, occ_mode,
-                                                                degen_tol, fermi_T, L);
+  const long long nt = (ns + 31) / 32;
+  k_loewner<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, st>>>(eps, occ, ns, mu, kT, occ_mode, degen_tol, fermi_T, L);
   return cudaGetLastError();
 }
 
