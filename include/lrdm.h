@@ -117,9 +117,9 @@ typedef struct lrdm_options {
   int poisson_symbol;    /* 0: 4 pi/|G|^2 (spectral); 1: second-order FD symbol  */
   int use_graph;         /* replay lrdm_gateaux_batch from a captured CUDA graph  */
   int autotune;          /* tensor-core precisions: 0 -> default launch shape
-                            (256 x 256 projection tiles on CTA pairs, response
-                            256-wide j-tiles over 256-row blocks on CTA pairs,
-                            direction group 4); 1 -> lrdm_create
+                            (projection on CTA pairs, two directions an item,
+                            response 256-wide j-tiles over 256-row blocks on
+                            CTA pairs, direction group 4); 1 -> lrdm_create
                             times the candidates (projection: pair tiles,
                             128 x 256 tiles, or 128 x 128 tiles with 1 or 2
                             directions; response: j-tile 128, 256
@@ -310,8 +310,9 @@ lrdm_status lrdm_profile_read(lrdm_ctx* ctx, double* gemm1_ms, long long* gemm1_
 
 /* Launch shape of the tensor-core contractions chosen at create (defaults
  * or the autotuner's choice): projection MMA width (128: square tiles; 256:
- * 128 x 256 tiles, one direction; 512: 256 x 256 tiles, one direction, each
- * computed by a pair of CTAs on neighbouring SMs with M = 256 pair MMAs),
+ * 128 x 256 tiles, one direction; 512: a pair of CTAs on neighbouring SMs with
+ * M = 256 pair MMAs over 128 rows x 256 columns of two directions, or 256 x 256
+ * of the last one of an odd number),
  * directions per projection square tile, response j-tile width (128, 256;
  * 512: 256-wide j-tiles over 256-row blocks on a CTA pair), response
  * direction group.  Any pointer may be NULL. */

@@ -2,12 +2,11 @@
 //
 // GEMM1  X_k[i, j] = sum_r (a_k[r] Psi[r, i]) Psi[r, j]     (H-breve', §II.C)
 //        upper-part tiles only; the whole grid reduction runs inside one
-//        tile, in segments of 1024 rows whose TMEM results are summed in FP32
-//        registers; the a_k weighting is applied to the A rows between their
+//        tile (or a row range of it), in segments of at most 1024 rows whose
+//        TMEM results are summed in FP32 registers; the a_k weighting is applied to the A rows between their
 //        TMA load and the MMAs, which read the weighted A from tensor memory.
-//        Three forms: 256 x 256 tiles on a CTA pair (cta_group::2, M = 256
-//        MMAs, each CTA holding half of the A and B rows; the default),
-//        128 x 256 tiles on one CTA, and 128 x 128 tiles with one or two
+//        Three forms: M = 256 MMAs on a CTA pair (cta_group::2; 128 rows x 256
+//        columns of two directions, one in each CTA; the default), 128 x 256 tiles on one CTA, and 128 x 128 tiles with one or two
 //        directions.
 // GEMM2  drho_k(r) = factor * sum_j Psi[r, j] (sum_{i <= j} Psi[r, i] X''_k[i, j])
 //        tile 128 (r) x 256 (j); for each j-block the i-reduction stops at the

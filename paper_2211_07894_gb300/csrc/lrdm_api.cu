@@ -499,7 +499,8 @@ lrdm_status tc_group(lrdm_ctx* ctx, int gemm, int out_is_io, cudaStream_t st) {
 // worth of start, last flush and tile store; the smallest count within half a
 // percent of the least, at least 128 stages a range.  48^3 / 512, K = 1 (3 items
 // for 76 pairs): 25 ranges, 228 -> 112 us against the former limit of 8; K = 2:
-// 12, 231 -> 180 us; K = 8 (24 items): 3; 96^3 / 4096, K = 16: 1.
+// 12, 231 -> 139 us with the two-direction items; K = 8 (20 items): 7, 491 us (3:
+// 540, 8: 642); 96^3 / 4096, K = 16: 1.
 int tc_split(long long items, long long units, int nch, int smax) {
   auto cost = [&](long long sp) {
     return (double)((items * sp + units - 1) / units) * ((double)nch / (double)sp + 100.0);

@@ -33,8 +33,8 @@ constexpr int G2_MAX_NJ = 64;
 
 // Launch shape of the tensor-core contractions (chosen by the autotuner or
 // the defaults): GEMM1 MMA width (128: square tiles with 1 or 2 directions;
-// 256: 128 x 256 tiles, one direction; G1_PAIR: 256 x 256 tiles, one
-// direction, on a CTA pair), directions per GEMM1 square tile,
+// 256: 128 x 256 tiles, one direction; G1_PAIR: 128 x 256 of two directions or
+// 256 x 256 of one on a CTA pair), directions per GEMM1 square tile,
 // GEMM2 j-tile width (128, 256; G2_PAIR: 256-wide j-tiles over 256-row
 // blocks on a CTA pair) and GEMM2 direction group (directions sharing one Psi
 // row block: 1, 2, 4).
