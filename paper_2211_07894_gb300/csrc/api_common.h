@@ -27,7 +27,10 @@ lrdm_status from_cufft(cufftResult r);
 bool release_idle();
 
 // Device allocation owned by the context (freed by lrdm_destroy), zeroed
-// unless zero == false.  A context has some 25 small buffers (up to 2 MB at
+// unless zero == false.  The zeroing is ordered on the stream of the set-up
+// (ctx->setup_st), which the create calls wait for before they return: on the
+// legacy stream it could run after the first kernels of a stream that does not
+// wait for that one, over what they had written.  A context has some 25 small buffers (up to 2 MB at
 // N_s = 512) beside the operand copies, each with its cudaMalloc, cudaMemset and
 // cudaFree: up to ARENA_MAX bytes they are cut from blocks of ARENA_BLOCK, which
 // are zeroed once (48^3, N_s = 512: create 1.75 -> 1.65 ms, destroy 1.06 -> 0.91
@@ -45,9 +48,7 @@ lrdm_status dalloc(lrdm_ctx* ctx, T** p, size_t count, bool zero = true) {
       void* q = nullptr;
       if (cudaMalloc(&q, ARENA_BLOCK) == cudaSuccess) {
         ctx->allocs.push_back(q);
-        // complete before work on other streams touches the block
-        LRDM_CU(cudaMemset(q, 0, ARENA_BLOCK));
-        LRDM_CU(cudaStreamSynchronize(cudaStreamLegacy));
+        LRDM_CU(cudaMemsetAsync(q, 0, ARENA_BLOCK, ctx->setup_st));
         ctx->arena = static_cast<char*>(q);
         ctx->arena_left = ARENA_BLOCK;
       } else {
@@ -70,7 +71,7 @@ lrdm_status dalloc(lrdm_ctx* ctx, T** p, size_t count, bool zero = true) {
   if (e != cudaSuccess) return from_cuda(e);
   ctx->allocs.push_back(q);
   if (zero) {
-    e = cudaMemset(q, 0, bytes);
+    e = cudaMemsetAsync(q, 0, bytes, ctx->setup_st);
     if (e != cudaSuccess) return from_cuda(e);
   }
   *p = static_cast<T*>(q);

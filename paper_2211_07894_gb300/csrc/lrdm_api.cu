@@ -280,15 +280,16 @@ lrdm_status setup_system(lrdm_ctx* ctx, int idx, const lrdm_system& in, cudaStre
   std::vector<std::vector<double>> eps(in.nspin), occ(in.nspin);
   for (int c = 0; c < in.nspin; ++c) {
     eps[c].resize(in.ns[c]);
-    LRDM_CU(cudaMemcpy(eps[c].data(), in.eps[c], in.ns[c] * sizeof(double),
-                       cudaMemcpyDeviceToHost));
+    LRDM_CU(cudaMemcpyAsync(eps[c].data(), in.eps[c], in.ns[c] * sizeof(double),
+                            cudaMemcpyDeviceToHost, st));
     if (S.occ_given) {
       if (!in.occ[c]) return LRDM_ERR_INVALID_ARG;
       occ[c].resize(in.ns[c]);
-      LRDM_CU(cudaMemcpy(occ[c].data(), in.occ[c], in.ns[c] * sizeof(double),
-                         cudaMemcpyDeviceToHost));
+      LRDM_CU(cudaMemcpyAsync(occ[c].data(), in.occ[c], in.ns[c] * sizeof(double),
+                              cudaMemcpyDeviceToHost, st));
     }
   }
+  LRDM_CU(cudaStreamSynchronize(st));
   lrdm_status ms = solve_mu_host(eps, S.ne, S.kT, S.g, &S.mu);
   if (ms != LRDM_OK) {
     if (!S.occ_given) return ms;
@@ -949,6 +950,7 @@ lrdm_status create_ctx(lrdm_ctx** out, const lrdm_system* sys, int nsys, const l
     return LRDM_ERR_OOM;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  ctx->setup_st = st;
   lrdm_status rc = LRDM_OK;
   do {
     if ((rc = dalloc(ctx, &ctx->d_status, 1)) != LRDM_OK) break;
@@ -1001,8 +1003,8 @@ lrdm_status create_ctx(lrdm_ctx** out, const lrdm_system* sys, int nsys, const l
       if ((rc = dalloc(ctx, reinterpret_cast<char**>(&ctx->tc_dev),
                        ctx->tc_host.size() * sizeof(TcProblem), false)) != LRDM_OK)
         break;
-      if (cudaMemcpy(ctx->tc_dev, ctx->tc_host.data(), ctx->tc_host.size() * sizeof(TcProblem),
-                     cudaMemcpyHostToDevice) != cudaSuccess) {
+      if (cudaMemcpyAsync(ctx->tc_dev, ctx->tc_host.data(), ctx->tc_host.size() * sizeof(TcProblem),
+                          cudaMemcpyHostToDevice, st) != cudaSuccess) {
         rc = LRDM_ERR_CUDA;
         break;
       }
@@ -1276,7 +1278,10 @@ lrdm_status lrdm_status_query(lrdm_ctx* ctx, int synchronize) {
   int h = 0;
   if (cudaMemcpy(&h, ctx->d_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
     return LRDM_ERR_CUDA;
-  if (cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess) return LRDM_ERR_CUDA;
+  // cleared before the next call's kernels on any stream
+  if (cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+    return LRDM_ERR_CUDA;
   if (h & STATUS_TIMEOUT) return LRDM_ERR_TIMEOUT;
   if (h & STATUS_NONFINITE) return LRDM_ERR_NONFINITE;
   if (h & STATUS_SINGULAR) return LRDM_ERR_SINGULAR;

@@ -189,6 +189,7 @@ struct lrdm_ctx {
   double* gs_scratch = nullptr;      // Gram-Schmidt partial sums (Krylov step)
   double* gs_norm = nullptr;         // [1] norm of the last normalised direction
   std::vector<void*> allocs;         // every device allocation, freed by lrdm_destroy
+  cudaStream_t setup_st = nullptr;   // stream of the set-up (create calls)
   char* arena = nullptr;             // rest of the last block of small buffers (dalloc)
   size_t arena_left = 0;
   // tensor-core problem table: one entry per (system, channel)

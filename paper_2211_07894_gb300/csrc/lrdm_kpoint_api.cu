@@ -257,7 +257,8 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
   ctx->kp_w.assign(in.k_weights, in.k_weights + nk);
   std::vector<std::vector<double>> eps(nk, std::vector<double>(ns)), occ(nk, std::vector<double>(ns));
   for (int q = 0; q < nk; ++q)
-    LRDM_CU(cudaMemcpy(eps[q].data(), in.eps[q], ns * sizeof(double), cudaMemcpyDeviceToHost));
+    LRDM_CU(cudaMemcpyAsync(eps[q].data(), in.eps[q], ns * sizeof(double), cudaMemcpyDeviceToHost, st));
+  LRDM_CU(cudaStreamSynchronize(st));
   LRDM_CK(solve_mu_kp_host(eps, ctx->kp_w, S.ne, S.kT, S.g, &S.mu));
   const size_t npsi = (size_t)S.Ng * ns, mat = (size_t)ns * ns;
   ctx->kp_C.assign(nk, nullptr);
@@ -362,8 +363,8 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
       ctx->tc_host.push_back(pr);
     }
     LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->tc_dev), ctx->tc_host.size() * sizeof(TcProblem), false));
-    LRDM_CU(cudaMemcpy(ctx->tc_dev, ctx->tc_host.data(), ctx->tc_host.size() * sizeof(TcProblem),
-                       cudaMemcpyHostToDevice));
+    LRDM_CU(cudaMemcpyAsync(ctx->tc_dev, ctx->tc_host.data(), ctx->tc_host.size() * sizeof(TcProblem),
+                            cudaMemcpyHostToDevice, st));
     ctx->tc_entries.reserve(nk);
   }
   LRDM_CU(cudaStreamSynchronize(st));   // the host eps / occ vectors end here
@@ -413,6 +414,7 @@ lrdm_status lrdm_kp_create(lrdm_ctx** out, const lrdm_kpoint_system* sys, const 
     return LRDM_ERR_OOM;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  ctx->setup_st = st;
   lrdm_status rc = LRDM_OK;
   do {
     if ((rc = dalloc(ctx, &ctx->d_status, 1)) != LRDM_OK) break;

@@ -114,6 +114,11 @@ lrdm_status lrdm_lrdma_create(lrdm_lrdma** out, long long n, int io_dtype, doubl
     lrdma_free(a);
     return rc;
   }
+  // the zeroing (legacy stream) is over before any stream uses the arrays
+  if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+    lrdma_free(a);
+    return LRDM_ERR_CUDA;
+  }
   a->U = u;
   a->T = t;
   a->R_lin = r;
