@@ -761,6 +761,18 @@ lrdm_status reduce_projections(lrdm_ctx* ctx, const int* K, bool adjoint, cudaSt
   return LRDM_OK;
 }
 
+// The directions of a forward call and the row ranges of its projections, which
+// the adjoint and lrdm_get_projection read X with.  A replayed graph runs no host
+// code, so its caller sets them too: another forward (a Krylov step) may have
+// run with other ranges since the capture.
+void set_forward(lrdm_ctx* ctx, const int* K) {
+  for (int s = 0; s < ctx->nsys; ++s) {
+    SysState& S = ctx->sys[s];
+    S.last_K = K[s];
+    if (K[s] > 0) S.nsplit = choose_split(ctx, s, K[s]);
+  }
+}
+
 lrdm_status forward_all(lrdm_ctx* ctx, const void* const* v, const int* K, void* const* f,
                         double* dmu_out, cudaStream_t st) {
   const int prec = ctx->opt.prec;
@@ -769,9 +781,9 @@ lrdm_status forward_all(lrdm_ctx* ctx, const void* const* v, const int* K, void*
   const size_t isz = io_size(io);
   const bool tc = is_tc(prec);
   const size_t csz = fp64 ? sizeof(double) : sizeof(float);
+  set_forward(ctx, K);
   for (int s = 0; s < ctx->nsys; ++s) {
     SysState& S = ctx->sys[s];
-    S.last_K = K[s];
     if (K[s] == 0) continue;
     LRDM_CK(gather_fields(ctx, S, K[s], st, [&](void* at, long long stride) {
       return launch_spin_sum(v[s], io, K[s], S.nspin, S.Ng, at, fp64, st, stride);
@@ -786,7 +798,6 @@ lrdm_status forward_all(lrdm_ctx* ctx, const void* const* v, const int* K, void*
   if (tc) {
     ctx->tc_entries.clear();
     for (int s = 0; s < ctx->nsys; ++s) {
-      if (K[s] > 0) ctx->sys[s].nsplit = choose_split(ctx, s, K[s]);
       for (int c = 0; c < ctx->sys[s].nspin && K[s] > 0; ++c) {
         TcEntry x = tc_entry(ctx, s, c, K[s]);
         x.X = ctx->sys[s].ch[c].Xpart;
@@ -796,11 +807,9 @@ lrdm_status forward_all(lrdm_ctx* ctx, const void* const* v, const int* K, void*
     }
     LRDM_CK(tc_group(ctx, 1, 0, st));
   } else {
-    for (int s = 0; s < ctx->nsys; ++s) {
-      if (K[s] > 0) ctx->sys[s].nsplit = choose_split(ctx, s, K[s]);
+    for (int s = 0; s < ctx->nsys; ++s)
       for (int c = 0; c < ctx->sys[s].nspin && K[s] > 0; ++c)
         LRDM_CK(gemm1_simt(ctx, ctx->sys[s], c, K[s], ctx->sys[s].ch[c].Xpart, st));
-    }
   }
   LRDM_CK(reduce_projections(ctx, K, false, st));
   // mu' and the Loewner scaling
@@ -1058,8 +1067,8 @@ lrdm_status lrdm_gateaux_batch(lrdm_ctx* ctx, const void* const* v, const int* K
       key.push_back(v[s]);
       key.push_back(f_out[s]);
       key.push_back(reinterpret_cast<const void*>((intptr_t)K[s]));
-      ctx->sys[s].last_K = K[s];
     }
+    set_forward(ctx, K);
     key.push_back(dmu_out);
     key.push_back(st);
     return graph_call(ctx, key, st, [&] { return forward_all(ctx, v, K, f_out, dmu_out, st); });
@@ -1195,8 +1204,7 @@ lrdm_status lrdm_backward(lrdm_ctx* ctx, const void* const* f_bar, void* const* 
   if (tc) {
     ctx->tc_entries.clear();
     for (int s = 0; s < ctx->nsys; ++s) {
-      // the same ranges as the forward call (the adjoint reduction reads X and Gbar together)
-      if (ctx->sys[s].last_K > 0) ctx->sys[s].nsplit = choose_split(ctx, s, ctx->sys[s].last_K);
+      // the forward call's ranges (the adjoint reduction reads X and Gbar together)
       for (int c = 0; c < ctx->sys[s].nspin && ctx->sys[s].last_K > 0; ++c) {
         TcEntry x = tc_entry(ctx, s, c, ctx->sys[s].last_K);
         x.X = ctx->sys[s].ch[c].Gpart;
