@@ -1,8 +1,11 @@
 // Element-wise and reduction kernels of the hot path: the perturbation
 // potential (Hartree symbol, LDA kernel, quadrature weight), the chemical-
 // potential shift mu' and the Loewner scaling of the projected matrices, and
-// the backward-only reductions.  All FP64 arithmetic where the result feeds an
-// FP64 quantity (mu', L, eps_bar, occ_bar).
+// the backward-only reductions.  mu', its adjoint's trace and the diagonals of
+// eps_bar and occ_bar are FP64 sums in every mode; FP32 partials of X and Gbar
+// over row ranges are added up as FP32 pairs (48 bits) before them, and the
+// off-diagonal entries of eps_bar and occ_bar are FP32 sums over the directions
+// where the partials are FP32 (k_eps_occ_bar).
 #include "lrdm_internal.h"
 
 #include <math.h>
@@ -260,33 +263,22 @@ struct DmuArgs {
   int K;
 };
 // num = sum_s sum_i L_ii X_ii and den = sum_s sum_i L_ii of direction k, valid
-// in thread 0.  FP32 partials (the FP32 and tensor-core modes) are summed and
-// multiplied as FP32 pairs: in FP64 the block's one SM, at two operations a
-// clock, took 13 to 30 us for what is one chain of load latencies.
-__device__ __forceinline__ void trace_sums(const DmuArgs& A, int k, int acc64, double& num, double& den) {
+// in thread 0, in FP64 in every mode: L_ii = -f_i (1 - f_i) / kT falls with the
+// exponential of the distance to mu and leaves the FP32 range where a gap is
+// wide.  FP32 partials of X are added up as FP32 pairs first.  Bound by the
+// latency of its strided loads and by the block's FP64 additions: 512 threads
+// where the partials are FP32 (N_s = 1024, seven ranges: 13 us; 256: 18, 1024: 14).
+template <typename T>
+constexpr int TRACE_THREADS = sizeof(T) == 8 ? 256 : 512;
+template <typename T>
+__device__ __forceinline__ void trace_sums(const DmuArgs& A, int k, double& num, double& den) {
   __shared__ double sn[32], sd[32];
-  __shared__ Pair32 sh[32];
-  if (!acc64) {
-    Pair32 n{0.f, 0.f}, d{0.f, 0.f};
-    for (int s = 0; s < A.nspin; ++s) {
-      const long long mat = (long long)A.ldx[s] * A.ldx[s];
-      for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
-        const Pair32 l = pair_split(A.L[s][(long long)i * A.ns[s] + i]);
-        const Pair32 x = sum_strided_pair(static_cast<const float*>(A.X[s]) + k * mat + (long long)i * A.ldx[s] + i,
-                                          A.nsplit, A.K * mat);
-        pair_fma(n, l, x);
-        pair_add(d, l);
-      }
-    }
-    num = pair_value(pair_block_sum(n, sh));
-    den = pair_value(pair_block_sum(d, sh));
-    return;
-  }
   num = den = 0.0;
   for (int s = 0; s < A.nspin; ++s) {
     const long long mat = (long long)A.ldx[s] * A.ldx[s];
+#pragma unroll 4
     for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
-      const double x = sum_strided(static_cast<const double*>(A.X[s]) + k * mat + (long long)i * A.ldx[s] + i,
+      const double x = sum_strided(static_cast<const T*>(A.X[s]) + k * mat + (long long)i * A.ldx[s] + i,
                                    A.nsplit, A.K * mat);
       const double l = A.L[s][(long long)i * A.ns[s] + i];
       num += l * x;
@@ -306,10 +298,11 @@ __device__ __forceinline__ void trace_sums(const DmuArgs& A, int k, int acc64, d
   }
 }
 
-__global__ void k_dmu(DmuArgs A, int acc64, double* __restrict__ dmu, double* __restrict__ dmu_out,
-                      int* __restrict__ status) {
+template <typename T>
+__global__ void __launch_bounds__(TRACE_THREADS<T>)
+    k_dmu(DmuArgs A, double* __restrict__ dmu, double* __restrict__ dmu_out, int* __restrict__ status) {
   double num, den;
-  trace_sums(A, blockIdx.x, acc64, num, den);
+  trace_sums<T>(A, blockIdx.x, num, den);
   if (threadIdx.x == 0) {
     const double m = den != 0.0 ? num / den : 0.0;
     if (!isfinite(m)) { atomicOr(status, STATUS_NONFINITE); }
@@ -413,9 +406,10 @@ __global__ void k_loewner_scale_tc(const float* __restrict__ X, int nsplit, int 
 
 // Backward trace terms T_k = sum_s sum_m L_mm Gbar_k,mm (the adjoint of the
 // mu' constraint) -- same reduction as k_dmu without the division.
-__global__ void k_trace_bar(DmuArgs A, int acc64, double* __restrict__ tbar) {
+template <typename T>
+__global__ void __launch_bounds__(TRACE_THREADS<T>) k_trace_bar(DmuArgs A, double* __restrict__ tbar) {
   double num, den;
-  trace_sums(A, blockIdx.x, acc64, num, den);
+  trace_sums<T>(A, blockIdx.x, num, den);
   if (threadIdx.x == 0) tbar[blockIdx.x] = num;
 }
 
@@ -753,14 +747,16 @@ static DmuArgs dmu_args(const SysState& S, const void* const* X, int K) {
 cudaError_t launch_dmu(const SysState& S, const void* const* Xparts, int K, int acc_fp64,
                        double* dmu, double* dmu_out, int* status, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  k_dmu<<<K, acc_fp64 ? 256 : 1024, 0, st>>>(dmu_args(S, Xparts, K), acc_fp64, dmu, dmu_out, status);
+  auto kern = acc_fp64 ? k_dmu<double> : k_dmu<float>;
+  kern<<<K, acc_fp64 ? TRACE_THREADS<double> : TRACE_THREADS<float>, 0, st>>>(dmu_args(S, Xparts, K), dmu, dmu_out, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_trace_bar(const SysState& S, const void* const* Gparts, int K, int acc_fp64,
                              double* tbar, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  k_trace_bar<<<K, acc_fp64 ? 256 : 1024, 0, st>>>(dmu_args(S, Gparts, K), acc_fp64, tbar);
+  auto kern = acc_fp64 ? k_trace_bar<double> : k_trace_bar<float>;
+  kern<<<K, acc_fp64 ? TRACE_THREADS<double> : TRACE_THREADS<float>, 0, st>>>(dmu_args(S, Gparts, K), tbar);
   return cudaGetLastError();
 }
 

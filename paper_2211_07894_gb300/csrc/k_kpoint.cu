@@ -17,55 +17,42 @@ namespace lrdm {
 namespace {
 
 // mu'_k over all k-points: one block per direction over all (point, state)
-// pairs; FP32 partials summed and multiplied as FP32 pairs (FP64 sums bound the
-// block's one SM).
-__global__ void __launch_bounds__(1024) k_kp_dmu(const __grid_constant__ KpDmuArgs A, double* __restrict__ dmu,
-                                                 double* __restrict__ dmu_out) {
-  __shared__ double sn[32], sd[32];
-  __shared__ Pair32 sh[32];
+// pairs, FP64 sums by as many threads as in trace_sums (k_elem.cu; 48^3, 4
+// points of 512: 12 us, 256 or 1024 threads 13 and 15).
+template <typename T>
+constexpr int KP_DMU_THREADS = sizeof(T) == 8 ? 256 : 512;
+template <typename T>
+__global__ void __launch_bounds__(KP_DMU_THREADS<T>)
+    k_kp_dmu(const __grid_constant__ KpDmuArgs A, double* __restrict__ dmu, double* __restrict__ dmu_out) {
+  constexpr int W = KP_DMU_THREADS<T> / 32;
+  __shared__ double sn[W], sd[W];
   const int k = blockIdx.x;
   const long long mat = (long long)A.ld * A.ld;
   double num = 0.0, den = 0.0;
-  Pair32 n{0.f, 0.f}, d{0.f, 0.f};
+#pragma unroll 4
   for (int e = threadIdx.x; e < A.nk * A.ns; e += blockDim.x) {
     const int kp = e / A.ns, i = e - kp * A.ns;
     const double l = A.kw[kp] * A.L[kp][(long long)i * A.ns + i];
-    const long long o = k * mat + (long long)i * A.ld + i, o2 = o + (long long)A.ns * A.ld + A.ns;
-    if (A.fp64) {
-      const double* P = static_cast<const double*>(A.P[kp]);
-      num += l * (sum_strided(P + o, A.nsplit, A.K * mat) + sum_strided(P + o2, A.nsplit, A.K * mat));
-      den += l;
-    } else {
-      const float* P = static_cast<const float*>(A.P[kp]);
-      Pair32 x = sum_strided_pair(P + o, A.nsplit, A.K * mat);
-      pair_add(x, sum_strided_pair(P + o2, A.nsplit, A.K * mat));
-      const Pair32 lp = pair_split(l);
-      pair_fma(n, lp, x);
-      pair_add(d, lp);
-    }
+    const T* P = static_cast<const T*>(A.P[kp]) + k * mat + (long long)i * A.ld + i;
+    num += l * (sum_strided(P, A.nsplit, A.K * mat) +
+                sum_strided(P + (long long)A.ns * A.ld + A.ns, A.nsplit, A.K * mat));
+    den += l;
   }
-  if (A.fp64) {
-    for (int o = 16; o > 0; o >>= 1) {
-      num += __shfl_xor_sync(0xffffffffu, num, o);
-      den += __shfl_xor_sync(0xffffffffu, den, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      sn[threadIdx.x >> 5] = num;
-      sd[threadIdx.x >> 5] = den;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      num = den = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        num += sn[w];
-        den += sd[w];
-      }
-    }
-  } else {
-    num = pair_value(pair_block_sum(n, sh));
-    den = pair_value(pair_block_sum(d, sh));
+  for (int o = 16; o > 0; o >>= 1) {
+    num += __shfl_xor_sync(0xffffffffu, num, o);
+    den += __shfl_xor_sync(0xffffffffu, den, o);
   }
+  if ((threadIdx.x & 31) == 0) {
+    sn[threadIdx.x >> 5] = num;
+    sd[threadIdx.x >> 5] = den;
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
+    num = den = 0.0;
+    for (int w = 0; w < W; ++w) {
+      num += sn[w];
+      den += sd[w];
+    }
     const double v = den != 0.0 ? num / den : 0.0;
     dmu[k] = v;
     if (dmu_out) dmu_out[k] = v;
@@ -306,7 +293,8 @@ inline unsigned kp_grid(long long n, int threads) {
 
 cudaError_t launch_kp_dmu(const KpDmuArgs& A, double* dmu, double* dmu_out, cudaStream_t st) {
   if (A.K == 0) return cudaSuccess;
-  k_kp_dmu<<<A.K, A.fp64 ? 256 : 1024, 0, st>>>(A, dmu, dmu_out);
+  auto kern = A.fp64 ? k_kp_dmu<double> : k_kp_dmu<float>;
+  kern<<<A.K, A.fp64 ? KP_DMU_THREADS<double> : KP_DMU_THREADS<float>, 0, st>>>(A, dmu, dmu_out);
   return cudaGetLastError();
 }
 

@@ -43,12 +43,6 @@ __device__ __forceinline__ Pair32 pair_split(double x) {
   const float h = (float)x;
   return Pair32{h, (float)(x - (double)h)};
 }
-// a += x y (both pairs; relative error about 2^-46)
-__device__ __forceinline__ void pair_fma(Pair32& a, const Pair32& x, const Pair32& y) {
-  const float p = __fmul_rn(x.s, y.s);
-  const float e = __fmaf_rn(x.s, y.c, __fmaf_rn(x.c, y.s, __fmaf_rn(x.s, y.s, -p)));
-  pair_add(a, Pair32{p, e});
-}
 __device__ __forceinline__ Pair32 pair_warp_sum(Pair32 a) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -56,17 +50,6 @@ __device__ __forceinline__ Pair32 pair_warp_sum(Pair32 a) {
   return a;
 }
 __device__ __forceinline__ double pair_value(const Pair32& a) { return (double)a.s + (double)a.c; }
-// Sum over the block (all threads call it), valid in every thread of warp 0.
-__device__ __forceinline__ Pair32 pair_block_sum(Pair32 a, Pair32* sh) {
-  a = pair_warp_sum(a);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
-  __syncthreads();
-  Pair32 r{0.f, 0.f};
-  if (threadIdx.x < (blockDim.x >> 5)) r = sh[threadIdx.x];
-  if (threadIdx.x < 32) r = pair_warp_sum(r);
-  __syncthreads();
-  return r;
-}
 __device__ __forceinline__ Pair32 sum_strided_pair(const float* __restrict__ p, int n, long long stride) {
   Pair32 x{p[0], 0.f};
 #pragma unroll 8
