@@ -116,16 +116,17 @@ __device__ __forceinline__ void dot4(Pair32& a, const float (&x)[4], const float
 // FP32 issue (ten operations a product).  At 96^3, K = 16: 84 us (50 us of issue),
 // against 378 us with one FP64 fma a product.
 //
-// FP32 range: a product's error word is exact while the values of a warp's
-// range stay below 2^60 and their largest is not below 2^-48 (its products'
-// last bits then stay above 2^-149; smaller values in the range lose less
-// than 2^-53 of the sum).  A warp whose range breaks this (or holds an
+// FP32 range: the sums stay finite while the values of a warp's range stay below
+// 2^56 (512 products a lane, 32 lanes: below 2^126), and a product's error word
+// is exact while their largest is not below 2^-48 (its products' last bits then
+// stay above 2^-149; smaller values in the range lose less than 2^-53 of the
+// sum).  A warp whose range breaks this (or holds an
 // infinity) repeats its range in FP64.
 constexpr int GR_WARPS = 8;
 constexpr int GR_RED = 160;                             // sums of 16 a block holds in shared memory
 constexpr int GR_TASKS = 153;                           // K = 64: 17 groups
 constexpr int GR_SEG = 128;                             // steps a lane sums in FP32 pairs (512 points)
-constexpr float GR_MAX = 1.152921504606846976e18f;      // 2^60
+constexpr float GR_MAX = 7.2057594037927936e16f;        // 2^56
 constexpr float GR_MIN = 3.552713678800501e-15f;        // 2^-48
 
 struct GramPlan {
