@@ -9,8 +9,11 @@
 // the grid-length sums of FP32 data run as compensated FP32 sums: products and
 // sums are split into value and rounding error (x y = p + e with
 // e = fma(x, y, -p); Knuth's two-sum), the errors summed in a second word
-// (the Dot2 algorithm of Ogita, Rump and Oishi, 2005), about 48 bits at ten
-// FP32 operations a product in place of one FP64 fma at 64 times the cost.
+// (the Dot2 algorithm of Ogita, Rump and Oishi, 2005), at eleven FP32 operations a
+// product in place of one FP64 fma at 64 times the cost.  A product and an
+// addition are good to about 2^-48.  The second word is itself an FP32 sum: left
+// to grow beside the first, its rounding grows with the square of the number of
+// terms, so it is folded back (dot4, UPD_NORM), and sums go to FP64 at GR_SEG.
 #include "lrdm_internal.h"
 
 #include <math.h>
@@ -88,7 +91,9 @@ constexpr long long LS_N32 = 65536;
 // rounding errors of products and of sums kept apart until the end: a square's
 // error word ends in fixed bits (x^2 = 1 mod 8), and dropping them one product
 // at a time against the growing sum biased <f, f> by 6e-15 (now 3e-16; FP64
-// sums: 1e-16 to 7e-16).
+// sums: 1e-16 to 7e-16).  The pair leaves renormalised: over 128 steps of constant
+// data the error of a lane's sum was 2e-12 without (above the default cutoff of
+// the pseudo-inverse), 7e-14 with it.
 __device__ __forceinline__ void dot4(Pair32& a, const float (&x)[4], const float (&y)[4]) {
   float p[4], e[4];
 #pragma unroll
@@ -100,10 +105,13 @@ __device__ __forceinline__ void dot4(Pair32& a, const float (&x)[4], const float
   two_sum(p[0], p[1], s01, r01);
   two_sum(p[2], p[3], s23, r23);
   two_sum(s01, s23, s, r);
-  two_sum(a.s, s, a.s, t);
+  float S;
+  two_sum(a.s, s, S, t);
   const float es = __fadd_rn(__fadd_rn(e[0], e[1]), __fadd_rn(e[2], e[3]));
   const float rs = __fadd_rn(__fadd_rn(r01, r23), __fadd_rn(r, t));
-  a.c = __fadd_rn(a.c, __fadd_rn(es, rs));
+  const float lo = __fadd_rn(a.c, __fadd_rn(es, rs));
+  a.s = __fadd_rn(S, lo);
+  a.c = __fsub_rn(lo, __fsub_rn(a.s, S));
 }
 
 // Gram sums of FP32 data.  The K + 1 vectors (f_0 .. f_{K-1}, R) are taken in
@@ -113,19 +121,25 @@ __device__ __forceinline__ void dot4(Pair32& a, const float (&x)[4], const float
 // from global memory (the block's other warps find them in L1).  The host
 // deals the tasks over 1, 2, 4 or 8 bins by their products (gram_plan); the
 // block's eight warps are that many bins times slices of the points.  Bound by
-// FP32 issue (ten operations a product).  At 96^3, K = 16: 84 us (50 us of issue),
-// against 378 us with one FP64 fma a product.
+// FP32 issue (eleven operations a product).  At 96^3, K = 16: 89 us (54 us of
+// issue; 85 us without the renormalisation), against 378 us with one FP64 fma a
+// product.
 //
 // FP32 range: the sums stay finite while the values of a warp's range stay below
-// 2^56 (512 products a lane, 32 lanes: below 2^126), and a product's error word
+// 2^56 (256 products a lane, 32 lanes: below 2^125), and a product's error word
 // is exact while their largest is not below 2^-48 (its products' last bits then
 // stay above 2^-149; smaller values in the range lose less than 2^-53 of the
-// sum).  A warp whose range breaks this (or holds an
-// infinity) repeats its range in FP64.
+// sum).  A warp whose range breaks this (or holds an infinity) repeats its range
+// in FP64.
 constexpr int GR_WARPS = 8;
 constexpr int GR_RED = 160;                             // sums of 16 a block holds in shared memory
 constexpr int GR_TASKS = 153;                           // K = 64: 17 groups
-constexpr int GR_SEG = 128;                             // steps a lane sums in FP32 pairs (512 points)
+// Steps a lane sums in FP32 pairs (256 points) before its sums go to FP64.  Relative
+// error of a lane's sum of positive products over 64 steps, largest of 400 draws:
+// random data 3e-14, data constant over the grid 5e-14 (6e-14 where lanes differ);
+// a warp's sums of random data are good to 1e-14 and average out over the warps
+// (884,736 points: 3e-16).  Sending them to FP64 costs four steps.
+constexpr int GR_SEG = 64;
 constexpr float GR_MAX = 7.2057594037927936e16f;        // 2^56
 constexpr float GR_MIN = 3.552713678800501e-15f;        // 2^-48
 
@@ -617,7 +631,7 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
                                                   const double* __restrict__ scal,
                                                   float* __restrict__ rho,
                                                   double* __restrict__ upd_partial) {
-  constexpr int UB = 4;
+  constexpr int UB = 4, UPD_NORM = 16;                  // directions a batch, and between renormalisations
   __shared__ float2 a[KMAX_LIMIT + UB];                 // zero past K
   __shared__ int se;
   __shared__ double sw[8];
@@ -642,6 +656,13 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
     const long long r0 = 2 * it;
     const bool two = r0 + 1 < n;
     Pair32 d[2] = {{0.f, 0.f}, {0.f, 0.f}}, fa[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    auto norm = [&] {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        pair_norm(fa[u]);
+        if (RHO) pair_norm(d[u]);
+      }
+    };
     if (vec) {
       // batches of UB directions, the next batch's loads in flight during a
       // batch's arithmetic (past K: coefficient 0, the last row again)
@@ -673,6 +694,7 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
             axpy2(d[1], c.x, c.y, wx[u].y);
           }
         }
+        if (k0 % UPD_NORM == UPD_NORM - UB) norm();
       }
     } else {
 #pragma unroll 4
@@ -685,6 +707,7 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
           axpy2(d[0], c.x, c.y, __ldg(v + o));
           axpy2(d[1], c.x, c.y, two ? __ldg(v + o + 1) : 0.f);
         }
+        if (k % UPD_NORM == UPD_NORM - 1) norm();
       }
     }
 #pragma unroll
@@ -716,6 +739,7 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
       if (isfinite(p) && isfinite(out)) {
         const float pe = __fmaf_rn(__fadd_rn(hi, hi), rl, __fmaf_rn(hi, hi, -p));
         pair_add(sq, Pair32{p, pe});
+        pair_norm(sq);
       } else {
         double dd = 0.0, ff = 0.0;
         for (int k = 0; k < K; ++k) {

@@ -39,6 +39,13 @@ __device__ __forceinline__ void pair_add(Pair32& a, const Pair32& b) {
   two_sum(a.s, b.s, a.s, r);
   a.c = __fadd_rn(a.c, __fadd_rn(b.c, r));
 }
+// The same value with the error word back below the rounding of the sum: a word
+// that collects the errors of many additions is itself rounded ever more coarsely.
+__device__ __forceinline__ void pair_norm(Pair32& a) {
+  const float s = __fadd_rn(a.s, a.c);
+  a.c = __fsub_rn(a.c, __fsub_rn(s, a.s));
+  a.s = s;
+}
 __device__ __forceinline__ Pair32 pair_split(double x) {
   const float h = (float)x;
   return Pair32{h, (float)(x - (double)h)};

@@ -1,11 +1,27 @@
-"""The least-squares step near the ends of the FP32 range: values just inside and
-outside the range in which its sums run as compensated FP32 pairs."""
+"""The least-squares step near the ends of the FP32 range and over long sums: values
+just inside and outside the range in which its sums run as compensated FP32 pairs,
+and constant data over many steps of a lane, where rounding errors do not
+average out."""
 
 import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
+
+
+def _apply(R, V, F, alpha, rho=None, w=0.125):
+    from paper_2211_07894_gb300 import binding
+    K, n = F.shape
+    coef = torch.empty(K, dtype=torch.float64, device="cuda")
+    srel = torch.empty(1, dtype=torch.float64, device="cuda")
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    code = binding.lrdm_apply_static(R.data_ptr(), V.data_ptr(), F.data_ptr(), binding.DTYPE_F32, K, n, w, alpha,
+                                     1e-12, rho.data_ptr() if rho is not None else 0, coef.data_ptr(),
+                                     srel.data_ptr(), status.data_ptr())
+    assert code == 0
+    torch.cuda.synchronize()
+    return coef, float(srel), int(status)
 
 
 def _context_apply(n, R, V, F, alpha, rho):
@@ -43,6 +59,44 @@ def test_gram_below_the_upper_end(size):
     a, s, status = _context_apply(n, R[None].contiguous(), V[:, None].contiguous(), F[:, None].contiguous(), 0.5, out)
     assert status == 0
     # random columns: condition below 2; 64 sums of products rounded to 2^-48
+    tol = 2.0 * 64 * 2.0 ** -48
+    assert float((a - a_ref).abs().max()) <= tol * max(1.0, float(a_ref.abs().max()))
+    assert abs(s - s_ref) <= tol * s_ref
+    assert float((out[0].double() - rho_ref).abs().max()) <= 2.0 ** -23 * float(rho_ref.abs().max())
+
+
+# 128 steps of every lane with one vector (eight slices): 128 * 128 * 304 * 8 points
+@pytest.mark.parametrize("c,d", [(0.7, 0.3), (1.1, 1.9), (0.37, 1.21), (1.7, 0.69)])
+def test_constant_columns(c, d):
+    """<f, R> / <f, f> of constant f and R.  A lane's pair is
+    renormalised at every step and summed over 64 steps at a time: an emulation of
+    one lane stays below 6e-14 for either sum, one running pair of 128 steps
+    reaches 2e-12."""
+    n = 128 * 128 * 304 * 8
+    F = torch.full((1, n), c, device="cuda")
+    R = torch.full((n,), d, device="cuda")
+    a, s, status = _apply(R, F, F, 0.5)
+    want = float(np.float64(np.float32(d)) / np.float64(np.float32(c)))
+    assert status == 0
+    assert abs(float(a[0]) - want) <= 1e-13 * want
+    assert s <= 1e-12
+
+
+@pytest.mark.parametrize("n", [(137, 136, 135), (137, 137, 137)])
+def test_second_segment_against_fp64(n):
+    """64 directions (one slice): a lane's points outgrow one segment (2.5 million
+    points)."""
+    ng = int(np.prod(n))
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n[0])
+    F = torch.randn(64, ng, generator=gen, device="cuda")
+    V = torch.randn(64, ng, generator=gen, device="cuda")
+    R = torch.randn(ng, generator=gen, device="cuda")
+    rho = torch.rand(ng, generator=gen, device="cuda")
+    a_ref, s_ref, rho_ref = _reference(R, V, F, rho, 0.5)
+    out = rho.clone()[None]
+    a, s, status = _context_apply(n, R[None], V[:, None].contiguous(), F[:, None].contiguous(), 0.5, out)
+    assert status == 0
     tol = 2.0 * 64 * 2.0 ** -48
     assert float((a - a_ref).abs().max()) <= tol * max(1.0, float(a_ref.abs().max()))
     assert abs(s - s_ref) <= tol * s_ref
