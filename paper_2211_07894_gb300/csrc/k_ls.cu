@@ -17,6 +17,7 @@
 #include "lrdm_internal.h"
 
 #include <math.h>
+#include <string.h>
 
 #include <atomic>
 
@@ -622,11 +623,23 @@ __device__ __forceinline__ void axpy2(Pair32& a, float h, float l, float x) {
 // stay in range; a point whose compensated sums leave the FP32 range (not
 // finite) is repeated in FP64.  At 96^3, K = 16 (124 MB to move: 19 us): 25 us,
 // against 127 us in FP64 (44 us with the loads in the K loop itself).
+constexpr int UPD_COEF = -96;                           // below 2^-96 a factor's second word is not normal
+constexpr double UPD_RMS2 = 6.842277657836020854e-49;   // 2^-160: an error word's 2^-149 is 2^-69 of rms(R)
+constexpr float UPD_OUT = 1.262177448353618888658765e-29f;                  // 2^-96
+
+// 0 < |x| < 2^e, in integer operations
+__host__ __device__ __forceinline__ bool below(double x, int e) {
+  uint64_t b;
+  memcpy(&b, &x, sizeof(b));
+  b <<= 1;
+  return b != 0 && b < (uint64_t)(1023 + e) << 53;
+}
+
 template <bool RHO>
 __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
                                                   const float* __restrict__ f,
                                                   const float* __restrict__ R, int K, long long n,
-                                                  double wn, int vec, double alpha,
+                                                  double wn, int vec, double alpha, int wide0,
                                                   const double* __restrict__ coef,
                                                   const double* __restrict__ scal,
                                                   float* __restrict__ rho,
@@ -635,16 +648,20 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
   __shared__ float2 a[KMAX_LIMIT + UB];                 // zero past K
   __shared__ int se;
   __shared__ double sw[8];
+  bool tiny = wide0 != 0;
   if (threadIdx.x < KMAX_LIMIT + UB) {
-    const Pair32 p = pair_split(threadIdx.x < K ? coef[threadIdx.x] : 0.0);
+    const double c = threadIdx.x < K ? coef[threadIdx.x] : 0.0;
+    const Pair32 p = pair_split(c);
     a[threadIdx.x] = make_float2(p.s, p.c);
+    tiny = tiny || below(c, UPD_COEF);
   }
   if (threadIdx.x == 128) {
     // 2^e near 1 / rms(R); e = 0 for R = 0 or not finite
     const double ms = scal[0] / wn;
     se = ms > 0.0 && isfinite(ms) ? max(-120, min(120, -ilogb(ms) / 2)) : 0;
+    tiny = tiny || (ms > 0.0 && ms < UPD_RMS2);
   }
-  __syncthreads();
+  const bool wide = __syncthreads_or(tiny);
   const Pair32 al = pair_split(alpha);
   const int e = se;
   const float sc = __int_as_float((127 + e) << 23);
@@ -736,7 +753,8 @@ __global__ void __launch_bounds__(256) k_update32(const float* __restrict__ v,
           out = __fadd_rn(d[u].s, d[u].c);
         }
       }
-      if (isfinite(p) && isfinite(out)) {
+      const bool low = RHO && fabsf(out) < UPD_OUT && d[u].s != 0.f;
+      if (!wide && !low && isfinite(p) && isfinite(out)) {
         const float pe = __fmaf_rn(__fadd_rn(hi, hi), rl, __fmaf_rn(hi, hi, -p));
         pair_add(sq, Pair32{p, pe});
         pair_norm(sq);
@@ -873,7 +891,7 @@ cudaError_t update_launch(const void* v, const void* f, const void* R, int io_dt
     auto kern = rho ? k_update32<true> : k_update32<false>;
     kern<<<UPD_BLOCKS, 256, 0, st>>>(static_cast<const float*>(v), static_cast<const float*>(f),
                                      static_cast<const float*>(R), K, n, w * (double)n, vec, alpha,
-                                     coef, scal, static_cast<float*>(rho), upd_partial);
+                                     (int)below(alpha, UPD_COEF), coef, scal, static_cast<float*>(rho), upd_partial);
   } else {
     k_update64<double><<<UPD_BLOCKS, 256, 0, st>>>(static_cast<const double*>(v),
                                                    static_cast<const double*>(f),

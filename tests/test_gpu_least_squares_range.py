@@ -1,6 +1,6 @@
 """The least-squares step near the ends of the FP32 range and over long sums: values
 just inside and outside the range in which its sums run as compensated FP32 pairs,
-and constant data over many steps of a lane, where rounding errors do not
+coefficients, residuals and densities far below 1, and constant data over many steps of a lane, where rounding errors do not
 average out."""
 
 import numpy as np
@@ -63,6 +63,35 @@ def test_gram_below_the_upper_end(size):
     assert float((a - a_ref).abs().max()) <= tol * max(1.0, float(a_ref.abs().max()))
     assert abs(s - s_ref) <= tol * s_ref
     assert float((out[0].double() - rho_ref).abs().max()) <= 2.0 ** -23 * float(rho_ref.abs().max())
+
+
+@pytest.mark.parametrize("f,r,v", [(1e-30, 1e-30, 1.0), (1.0, 1e-32, 1e30), (1e25, 1e-18, 1e30), (1e20, 1e-20, 1e35),
+                                   (1e-3, 1e-28, 1.0), (1.0, 1.0, 1e-37)])
+@pytest.mark.parametrize("n", [68921, 68880])
+def test_update_far_below_one(f, r, v, n):
+    """Coefficients of r / f and residuals of size r: s_rel keeps the accuracy it has
+    at size 1, the density its FP32 rounding."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(9)
+    K = 5
+    F = torch.randn(K, n, generator=gen, device="cuda") * f
+    R = torch.randn(n, generator=gen, device="cuda") * r
+    V = torch.randn(K, n, generator=gen, device="cuda") * v
+    size = v * r / f
+    for alpha in (0.5, 0.0):
+        rho = torch.rand(n, generator=gen, device="cuda") * size
+        a_ref, s_ref, rho_ref = _reference(R, V, F, rho, alpha)
+        if alpha == 0.0:
+            rho_ref = a_ref @ V.double()
+        out = rho.clone()
+        a, s, status = _apply(R, V, F, alpha, out)
+        assert status == 0
+        tol = 2.0 * 8 * 2.0 ** -48                # as for data of size 1
+        assert float((a - a_ref).abs().max()) <= tol * max(r / f, float(a_ref.abs().max()))
+        assert abs(s - s_ref) <= tol * s_ref
+        # FP32 rounding, the coefficients' error, half the spacing of the denormals
+        err = (out.double() - rho_ref).abs()
+        assert bool((err <= 2.0 ** -23 * rho_ref.abs() + 2.0 ** -35 * float(rho_ref.abs().max()) + 2.0 ** -149).all())
 
 
 # 128 steps of every lane with one vector (eight slices): 128 * 128 * 304 * 8 points
