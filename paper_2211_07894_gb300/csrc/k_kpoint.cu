@@ -209,11 +209,11 @@ __global__ void __launch_bounds__(128) k_kp_scale_tc(const float* __restrict__ P
         if (c0 + e > j) continue;
         const Pair32 x = xs[e];
         if (c0 + e == j) {
-          v[e] = (float)(ld64 * ((double)x.s + (double)x.c - (j < n2 ? dmu[k] : 0.0)));
+          v[e] = (float)(ld64 * (pair_value(x) - (j < n2 ? dmu[k] : 0.0)));
         } else {
           const float q = __fmul_rn(l[e].s, x.s);
           const float qe = __fmaf_rn(l[e].c, x.s, __fmaf_rn(l[e].s, x.c, __fmaf_rn(l[e].s, x.s, -q)));
-          v[e] = __fadd_rn(q, qe);
+          v[e] = pair_round(Pair32{q, qe});
         }
       }
     }
@@ -249,6 +249,12 @@ __device__ __forceinline__ Pair32 kp_parts(const KpSumArgs& A, long long o) {
   for (int q = 1; q < A.nk; ++q) pair_add(d, Pair32{A.part[q][o], 0.f});
   return d;
 }
+// The same in FP64, where the pair's sum has left the FP32 range.
+__device__ __noinline__ double kp_parts64(const KpSumArgs& A, long long o) {
+  double x = 0.0;
+  for (int q = 0; q < A.nk; ++q) x += (double)A.part[q][o];
+  return x;
+}
 
 // f = sum_kappa part_kappa - v
 __global__ void k_kp_sum(const __grid_constant__ KpSumArgs A, const void* __restrict__ v, int io, long long n,
@@ -257,10 +263,13 @@ __global__ void k_kp_sum(const __grid_constant__ KpSumArgs A, const void* __rest
        e += (long long)gridDim.x * blockDim.x) {
     Pair32 d = kp_parts(A, e);
     if (io == LRDM_DTYPE_F64) {
-      static_cast<double*>(f)[e] = (double)d.s + (double)d.c - static_cast<const double*>(v)[e];
+      const double x = isfinite(d.s) ? pair_value(d) : kp_parts64(A, e);
+      static_cast<double*>(f)[e] = x - static_cast<const double*>(v)[e];
     } else {
-      pair_add(d, Pair32{-static_cast<const float*>(v)[e], 0.f});
-      static_cast<float*>(f)[e] = __fadd_rn(d.s, d.c);
+      const float ve = static_cast<const float*>(v)[e];
+      const bool in = isfinite(d.s);
+      pair_add(d, Pair32{-ve, 0.f});
+      static_cast<float*>(f)[e] = in ? pair_round(d) : (float)(kp_parts64(A, e) - (double)ve);
     }
   }
 }
@@ -275,12 +284,17 @@ __global__ void k_kp_collect(const __grid_constant__ KpSumArgs A, int use_parts,
   if (r >= ld) return;
   Pair32 d{0.f, 0.f};
   double d64 = 0.0;
+  bool pair = use_parts;
   if (r < Ng) {
     if (use_parts) d = kp_parts(A, k * Ng + r);
     else d64 = drho[k * Ng + r];
+    if (use_parts && !isfinite(d.s)) {
+      d64 = kp_parts64(A, k * Ng + r);
+      pair = false;
+    }
   }
-  if (fp64) static_cast<double*>(out)[k * ld + r] = use_parts ? (double)d.s + (double)d.c : d64;
-  else static_cast<float*>(out)[k * ld + r] = use_parts ? __fadd_rn(d.s, d.c) : (float)d64;
+  if (fp64) static_cast<double*>(out)[k * ld + r] = pair ? pair_value(d) : d64;
+  else static_cast<float*>(out)[k * ld + r] = pair ? pair_round(d) : (float)d64;
 }
 
 inline unsigned kp_grid(long long n, int threads) {

@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(F32Cfg<T>::THREADS, F32Cfg<T>::BLOCKS)
   double tot[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
-    double p = (double)ps[m].s + (double)ps[m].c;
+    double p = pair_value(ps[m]);
     for (int s = 4; s > 0; s >>= 1) p += __shfl_xor_sync(0xffffffffu, p, s);
     tot[m] = p;
     if (wc == 64 && (lane & 7) == 0) red[wr + f32_row(lane, m)] = p;

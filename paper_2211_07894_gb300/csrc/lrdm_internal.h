@@ -56,7 +56,12 @@ __device__ __forceinline__ Pair32 pair_warp_sum(Pair32 a) {
     pair_add(a, Pair32{__shfl_xor_sync(0xffffffffu, a.s, o), __shfl_xor_sync(0xffffffffu, a.c, o)});
   return a;
 }
-__device__ __forceinline__ double pair_value(const Pair32& a) { return (double)a.s + (double)a.c; }
+// The value in FP64, and rounded to FP32.  The first word of a sum that left the
+// FP32 range is its infinity or NaN, the error word a NaN either way.
+__device__ __forceinline__ double pair_value(const Pair32& a) {
+  return isfinite(a.s) ? (double)a.s + (double)a.c : (double)a.s;
+}
+__device__ __forceinline__ float pair_round(const Pair32& a) { return isfinite(a.s) ? __fadd_rn(a.s, a.c) : a.s; }
 __device__ __forceinline__ Pair32 sum_strided_pair(const float* __restrict__ p, int n, long long stride) {
   Pair32 x{p[0], 0.f};
 #pragma unroll 8
