@@ -319,8 +319,8 @@ template <typename Tc>
 __global__ void k_loewner_scale(const Tc* __restrict__ X, int nsplit, int K, int ns,
                                 const double* __restrict__ L, const double* __restrict__ shift,
                                 int adjoint, double inv_trace, Tc* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = blockIdx.y, k = blockIdx.z;
+  const int j = blockIdx.y * blockDim.x + threadIdx.x;
+  const int i = blockIdx.x, k = blockIdx.z;            // rows in x: a grid's y ends at 65,535
   if (j >= ns || j < i) return;
   const long long mat = (long long)ns * ns, o = (long long)k * mat + (long long)i * ns + j;
   const double x = sum_strided(X + o, nsplit, (long long)K * mat);
@@ -775,7 +775,7 @@ cudaError_t launch_loewner_scale(const SysState& S, int s, const void* Xpart, in
                                               static_cast<__nv_bfloat16*>(c.Xpp_lo));
     return cudaGetLastError();
   }
-  const dim3 grid((unsigned)((c.ns + 127) / 128), (unsigned)c.ns, (unsigned)K);
+  const dim3 grid((unsigned)c.ns, (unsigned)((c.ns + 127) / 128), (unsigned)K);
   if (acc_fp64)
     k_loewner_scale<double><<<grid, 128, 0, st>>>(static_cast<const double*>(Xpart), S.nsplit, K, c.ns, c.L,
                                                   shift, adjoint, inv_trace_L, static_cast<double*>(c.Xpp));

@@ -67,8 +67,8 @@ __global__ void k_kp_scale(const Tc* __restrict__ P, int nsplit, int K, int ns,
                            const double* __restrict__ L, const double* __restrict__ dmu,
                            Tc* __restrict__ Y) {
   const int n2 = 2 * ns;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = blockIdx.y, k = blockIdx.z;
+  const int j = blockIdx.y * blockDim.x + threadIdx.x;
+  const int i = blockIdx.x, k = blockIdx.z;            // rows in x: a grid's y ends at 65,535
   if (j >= n2 || i > j) return;
   const long long mat = (long long)n2 * n2, tot = (long long)K * mat;
   const Tc* Pk = P + (long long)k * mat;
@@ -315,7 +315,7 @@ cudaError_t launch_kp_dmu(const KpDmuArgs& A, double* dmu, double* dmu_out, cuda
 cudaError_t launch_kp_scale(int fp64, const void* P, int nsplit, int K, int ns, const double* L,
                             const double* dmu, void* Y, cudaStream_t st) {
   if (K == 0) return cudaSuccess;
-  const dim3 grid((unsigned)((2 * ns + 127) / 128), (unsigned)(2 * ns), (unsigned)K);
+  const dim3 grid((unsigned)(2 * ns), (unsigned)((2 * ns + 127) / 128), (unsigned)K);
   if (fp64)
     k_kp_scale<double><<<grid, 128, 0, st>>>(static_cast<const double*>(P), nsplit, K, ns, L, dmu,
                                              static_cast<double*>(Y));
