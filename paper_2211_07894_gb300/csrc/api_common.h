@@ -25,6 +25,9 @@ lrdm_status from_cufft(cufftResult r);
 
 // Destroys the plans kept from closed contexts; whether there were any.
 bool release_idle();
+// cudaMalloc, again without those plans where memory is short; a refusal leaves
+// no pending CUDA error behind (the create calls try again with less).
+lrdm_status device_alloc(void** q, size_t bytes);
 
 // Device allocation owned by the context (freed by lrdm_destroy), zeroed
 // unless zero == false.  The zeroing is ordered on the stream of the set-up
@@ -34,7 +37,8 @@ bool release_idle();
 // N_s = 512) beside the operand copies, each with its cudaMalloc, cudaMemset and
 // cudaFree: up to ARENA_MAX bytes they are cut from blocks of ARENA_BLOCK, which
 // are zeroed once (48^3, N_s = 512: create 1.75 -> 1.65 ms, destroy 1.06 -> 0.91
-// ms; the rest of both is the large buffers, 0.5 us a MB to free).
+// ms; the rest of both is the large buffers, 0.5 us a MB to free).  A context
+// made where memory is short (ctx->lean) has no blocks.
 constexpr size_t ARENA_BLOCK = 8u << 20, ARENA_MAX = 2u << 20, ARENA_ALIGN = 512;
 
 template <typename T>
@@ -42,7 +46,7 @@ lrdm_status dalloc(lrdm_ctx* ctx, T** p, size_t count, bool zero = true) {
   *p = nullptr;
   if (count == 0) count = 1;
   const size_t bytes = count * sizeof(T);
-  if (bytes <= ARENA_MAX) {
+  if (bytes <= ARENA_MAX && !ctx->lean) {
     const size_t need = (bytes + ARENA_ALIGN - 1) / ARENA_ALIGN * ARENA_ALIGN;
     if (need > ctx->arena_left) {
       void* q = nullptr;
@@ -63,17 +67,9 @@ lrdm_status dalloc(lrdm_ctx* ctx, T** p, size_t count, bool zero = true) {
     }
   }
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, bytes);
-  if (e == cudaErrorMemoryAllocation && release_idle()) {
-    (void)cudaGetLastError();
-    e = cudaMalloc(&q, bytes);
-  }
-  if (e != cudaSuccess) return from_cuda(e);
+  LRDM_CK(device_alloc(&q, bytes));
   ctx->allocs.push_back(q);
-  if (zero) {
-    e = cudaMemsetAsync(q, 0, bytes, ctx->setup_st);
-    if (e != cudaSuccess) return from_cuda(e);
-  }
+  if (zero) LRDM_CU(cudaMemsetAsync(q, 0, bytes, ctx->setup_st));
   *p = static_cast<T*>(q);
   return LRDM_OK;
 }

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(KP_DMU_THREADS<T>)
 // it the buffer keeps the zeros it was created with), summed over the row ranges.  P and L
 // are symmetric, so every read takes the entry whose column follows j.
 template <typename Tc>
-__global__ void k_kp_scale(const Tc* __restrict__ P, int nsplit, int K, int ns,
+__global__ void k_kp_scale(const Tc* __restrict__ P, int nsplit, int K, int k0, int ns,
                            const double* __restrict__ L, const double* __restrict__ dmu,
                            Tc* __restrict__ Y) {
   const int n2 = 2 * ns;
@@ -71,12 +71,12 @@ __global__ void k_kp_scale(const Tc* __restrict__ P, int nsplit, int K, int ns,
   const int i = blockIdx.x, k = blockIdx.z;            // rows in x: a grid's y ends at 65,535
   if (j >= n2 || i > j) return;
   const long long mat = (long long)n2 * n2, tot = (long long)K * mat;
-  const Tc* Pk = P + (long long)k * mat;
+  const Tc* Pk = P + (long long)(k0 + k) * mat;
   auto at = [&](int r, int c) { return sum_strided(Pk + (long long)r * n2 + c, nsplit, tot); };
   const int a = i < ns ? i : i - ns, b = j < ns ? j : j - ns;
   const double l = L[(long long)a * ns + b];
   double m;
-  if ((i < ns) == (j < ns)) m = l * (at(a, b) + at(ns + a, ns + b) - (a == b ? dmu[k] : 0.0));
+  if ((i < ns) == (j < ns)) m = l * (at(a, b) + at(ns + a, ns + b) - (a == b ? dmu[k0 + k] : 0.0));
   else m = l * (at(a, ns + b) - at(ns + a, b));          // Im X_ab = P12 - P21
   Y[(long long)k * mat + (long long)i * n2 + j] = (Tc)(i < j ? 2.0 * m : m);
 }
@@ -312,15 +312,15 @@ cudaError_t launch_kp_dmu(const KpDmuArgs& A, double* dmu, double* dmu_out, cuda
   return cudaGetLastError();
 }
 
-cudaError_t launch_kp_scale(int fp64, const void* P, int nsplit, int K, int ns, const double* L,
-                            const double* dmu, void* Y, cudaStream_t st) {
-  if (K == 0) return cudaSuccess;
-  const dim3 grid((unsigned)(2 * ns), (unsigned)((2 * ns + 127) / 128), (unsigned)K);
+cudaError_t launch_kp_scale(int fp64, const void* P, int nsplit, int K, int k0, int kn, int ns,
+                            const double* L, const double* dmu, void* Y, cudaStream_t st) {
+  if (kn == 0) return cudaSuccess;
+  const dim3 grid((unsigned)(2 * ns), (unsigned)((2 * ns + 127) / 128), (unsigned)kn);
   if (fp64)
-    k_kp_scale<double><<<grid, 128, 0, st>>>(static_cast<const double*>(P), nsplit, K, ns, L, dmu,
+    k_kp_scale<double><<<grid, 128, 0, st>>>(static_cast<const double*>(P), nsplit, K, k0, ns, L, dmu,
                                              static_cast<double*>(Y));
   else
-    k_kp_scale<float><<<grid, 128, 0, st>>>(static_cast<const float*>(P), nsplit, K, ns, L, dmu,
+    k_kp_scale<float><<<grid, 128, 0, st>>>(static_cast<const float*>(P), nsplit, K, k0, ns, L, dmu,
                                             static_cast<float*>(Y));
   return cudaGetLastError();
 }

@@ -208,6 +208,16 @@ PlanPool& plan_pool() {
 }
 bool release_idle() { return plan_pool().clear(); }
 
+lrdm_status device_alloc(void** q, size_t bytes) {
+  cudaError_t e = cudaMalloc(q, bytes);
+  if (e == cudaErrorMemoryAllocation && release_idle()) {
+    (void)cudaGetLastError();
+    e = cudaMalloc(q, bytes);
+  }
+  if (e == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+  return from_cuda(e);
+}
+
 PlanPool::Key plan_key(const SysState& S) {
   PlanPool::Key k;
   k.ctx = S.plan_ctx;
@@ -362,7 +372,7 @@ lrdm_status setup_system(lrdm_ctx* ctx, int idx, const lrdm_system& in, cudaStre
   // subspace) can split their grid reduction (CUDA cores: the count simt_split
   // takes; row-sharded: one per rank)
   S.xslots = S.kmax;
-  {
+  if (!ctx->lean) {
     size_t ldmax = 0;
     for (int c = 0; c < in.nspin; ++c)
       ldmax = std::max(ldmax, (size_t)(is_tc(prec) ? S.ch[c].ns_pad : S.ch[c].ns));
@@ -919,29 +929,12 @@ const char* lrdm_status_string(lrdm_status s) {
 }
 
 namespace {
-lrdm_status create_ctx(lrdm_ctx** out, const lrdm_system* sys, int nsys, const lrdm_options* opt,
-                       void* stream, const lrdm_rows* rows) {
-  if (!out) return LRDM_ERR_INVALID_ARG;
-  *out = nullptr;
-  if (!sys || nsys < 1) return LRDM_ERR_INVALID_ARG;
-  lrdm_options o;
-  if (opt) o = *opt;
-  else lrdm_default_options(&o);
-  if (o.prec < LRDM_FP64 || o.prec > LRDM_BF16X3) return LRDM_ERR_INVALID_ARG;
-  if (o.io_dtype != LRDM_DTYPE_F64 && o.io_dtype != LRDM_DTYPE_F32) return LRDM_ERR_INVALID_ARG;
-  if (o.k_max < 1 || o.k_max > KMAX_LIMIT) return LRDM_ERR_INVALID_ARG;
-  if (!(o.pinv_rcond >= 0.0)) return LRDM_ERR_INVALID_ARG;
-  if (!(o.degen_tol >= 0.0)) return LRDM_ERR_INVALID_ARG;
-  if (o.poisson_symbol != 0 && o.poisson_symbol != 1) return LRDM_ERR_INVALID_ARG;
-  if (o.fermi_T < 0 || o.fermi_T > 30) return LRDM_ERR_INVALID_ARG;
-  if (o.fermi_T > 0)
-    for (int s = 0; s < nsys; ++s)
-      if (sys[s].occ[0]) return LRDM_ERR_INVALID_ARG;
-  for (int s = 0; s < nsys; ++s) LRDM_CK(validate_system(sys[s], o));
-  if (is_tc(o.prec) && !tc_supported()) return LRDM_ERR_UNSUPPORTED;
-
+// A context of the validated systems (lean: with the least memory).
+lrdm_status make_ctx(lrdm_ctx** out, const lrdm_system* sys, int nsys, const lrdm_options& o, void* stream,
+                     const lrdm_rows* rows, bool lean) {
   lrdm_ctx* ctx = new (std::nothrow) lrdm_ctx();
   if (!ctx) return LRDM_ERR_OOM;
+  ctx->lean = lean;
   ctx->nsys = nsys;
   ctx->opt = o;
   if (rows) {
@@ -1029,6 +1022,32 @@ lrdm_status create_ctx(lrdm_ctx** out, const lrdm_system* sys, int nsys, const l
   }
   *out = ctx;
   return LRDM_OK;
+}
+
+// Checks the arguments; the buffers that only buy speed (several row ranges,
+// blocks of small buffers) are left out where everything does not fit.
+lrdm_status create_ctx(lrdm_ctx** out, const lrdm_system* sys, int nsys, const lrdm_options* opt,
+                       void* stream, const lrdm_rows* rows) {
+  if (!out) return LRDM_ERR_INVALID_ARG;
+  *out = nullptr;
+  if (!sys || nsys < 1) return LRDM_ERR_INVALID_ARG;
+  lrdm_options o;
+  if (opt) o = *opt;
+  else lrdm_default_options(&o);
+  if (o.prec < LRDM_FP64 || o.prec > LRDM_BF16X3) return LRDM_ERR_INVALID_ARG;
+  if (o.io_dtype != LRDM_DTYPE_F64 && o.io_dtype != LRDM_DTYPE_F32) return LRDM_ERR_INVALID_ARG;
+  if (o.k_max < 1 || o.k_max > KMAX_LIMIT) return LRDM_ERR_INVALID_ARG;
+  if (!(o.pinv_rcond >= 0.0)) return LRDM_ERR_INVALID_ARG;
+  if (!(o.degen_tol >= 0.0)) return LRDM_ERR_INVALID_ARG;
+  if (o.poisson_symbol != 0 && o.poisson_symbol != 1) return LRDM_ERR_INVALID_ARG;
+  if (o.fermi_T < 0 || o.fermi_T > 30) return LRDM_ERR_INVALID_ARG;
+  if (o.fermi_T > 0)
+    for (int s = 0; s < nsys; ++s)
+      if (sys[s].occ[0]) return LRDM_ERR_INVALID_ARG;
+  for (int s = 0; s < nsys; ++s) LRDM_CK(validate_system(sys[s], o));
+  if (is_tc(o.prec) && !tc_supported()) return LRDM_ERR_UNSUPPORTED;
+  const lrdm_status rc = make_ctx(out, sys, nsys, o, stream, rows, false);
+  return rc == LRDM_ERR_OOM ? make_ctx(out, sys, nsys, o, stream, rows, true) : rc;
 }
 }  // namespace
 

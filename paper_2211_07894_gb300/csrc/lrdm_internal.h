@@ -185,6 +185,8 @@ struct lrdm_ctx {
   double* gs_norm = nullptr;         // [1] norm of the last normalised direction
   std::vector<void*> allocs;         // every device allocation, freed by lrdm_destroy
   cudaStream_t setup_st = nullptr;   // stream of the set-up (create calls)
+  bool lean = false;                 // made where memory is short: one row range, no blocks,
+                                     // one X'' for all k-points (CUDA cores)
   char* arena = nullptr;             // rest of the last block of small buffers (dalloc)
   size_t arena_left = 0;
   // tensor-core problem table: one entry per (system, channel)
@@ -217,7 +219,9 @@ struct lrdm_ctx {
   std::vector<void*> kp_C;           // CUDA cores: [nk] stacked C = [Re Psi, Im Psi], [N_g][2 N_s]
   std::vector<double*> kp_eps, kp_occ, kp_L;
   std::vector<void*> kp_P;           // [nk] [xslots][2 N_s][2 N_s]: C^T diag(a) C
-  std::vector<void*> kp_Y;           // [nk] [kmax][2 N_s][2 N_s] Loewner-scaled
+  std::vector<void*> kp_Y;           // [nk] [kmax][2 N_s][2 N_s] Loewner-scaled; lean: the
+                                     // points' common buffer of kp_ydirs directions
+  int kp_ydirs = 0;
   double* kp_drho = nullptr;         // [kmax][N_g] FP64 accumulator
   // tensor-core modes: per k-point the stacked real operand C = [Re Psi, Im Psi]
   // (N_g x 2 N_s) as one channel of the real contractions, its problem index
@@ -261,8 +265,9 @@ struct KpSumArgs {
 cudaError_t launch_kp_dmu(const KpDmuArgs& A, double* dmu, double* dmu_out, cudaStream_t st);
 // CUDA-core modes: M'' [K][2 N_s][2 N_s] (upper part, compute type) from the
 // stacked Gram P [nsplit][K][2 N_s][2 N_s]
-cudaError_t launch_kp_scale(int fp64, const void* P, int nsplit, int K, int ns, const double* L,
-                            const double* dmu, void* Y, cudaStream_t st);
+// (directions k0 .. k0 + kn - 1 of K, into Y's first kn)
+cudaError_t launch_kp_scale(int fp64, const void* P, int nsplit, int K, int k0, int kn, int ns,
+                            const double* L, const double* dmu, void* Y, cudaStream_t st);
 cudaError_t launch_kp_finish(const double* drho, const void* v, int io, long long n, void* f,
                              cudaStream_t st);
 cudaError_t launch_kp_density(int fp64, const void* pr, const void* pi, int ns, int ld, long long Ng,

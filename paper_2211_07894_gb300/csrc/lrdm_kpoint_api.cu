@@ -147,19 +147,35 @@ lrdm_status kp_response(lrdm_ctx* ctx, int K, double factor, double* dmu_out, cu
     LRDM_CK(tc_group(ctx, 2, 0, st));
   } else {
     LRDM_CU(cudaMemsetAsync(ctx->kp_drho, 0, (size_t)K * S.Ng * sizeof(double), st));
-    for (int q = 0; q < nk; ++q)
-      LRDM_CU(launch_kp_scale(fp64, ctx->kp_P[q], split, K, ns, ctx->kp_L[q], S.dmu, ctx->kp_Y[q], st));
-    int pi = prof_begin(ctx, 2, st);
-    for (int q = 0; q < nk; ++q) {
+    // directions k0 .. k0 + kn - 1 of point q
+    auto scale = [&](int q, int k0, int kn) {
+      count(ctx, 1);
+      return launch_kp_scale(fp64, ctx->kp_P[q], split, K, k0, kn, ns, ctx->kp_L[q], S.dmu, ctx->kp_Y[q], st);
+    };
+    auto respond = [&](int q, int k0, int kn) {
       SimtOut o;
       o.mode = SIMT_OUT_ADD;
       o.factor = factor * ctx->kp_w[q];
-      o.out = ctx->kp_drho;
+      o.out = ctx->kp_drho + (size_t)k0 * S.Ng;
       o.stride = S.Ng;
-      LRDM_CU(launch_gemm2_simt(fp64, ctx->kp_C[q], 2 * ns, S.Ng, ctx->kp_Y[q], K, o, st));
+      count(ctx, 1);
+      return launch_gemm2_simt(fp64, ctx->kp_C[q], 2 * ns, S.Ng, ctx->kp_Y[q], kn, o, st);
+    };
+    if (!ctx->lean) {
+      for (int q = 0; q < nk; ++q) LRDM_CU(scale(q, 0, K));
+      const int pi = prof_begin(ctx, 2, st);
+      for (int q = 0; q < nk; ++q) LRDM_CU(respond(q, 0, K));
+      prof_end(ctx, pi, st);
+    } else {
+      for (int q = 0; q < nk; ++q)
+        for (int k0 = 0; k0 < K; k0 += ctx->kp_ydirs) {
+          const int kn = std::min(ctx->kp_ydirs, K - k0);
+          LRDM_CU(scale(q, k0, kn));
+          const int pi = prof_begin(ctx, 2, st);
+          LRDM_CU(respond(q, k0, kn));
+          prof_end(ctx, pi, st);
+        }
     }
-    prof_end(ctx, pi, st);
-    count(ctx, 2 * nk);
   }
   return LRDM_OK;
 }
@@ -279,12 +295,15 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
   if (!tc) {
     // partial Grams within 512 MB per point
     const int room = (int)std::min<size_t>(64, std::max<size_t>(1, (512ull << 20) / (S.kmax * mat2 * csz)));
-    S.xslots = simt_split(fp64, 2 * ns, S.Ng, S.kmax, room * S.kmax) * S.kmax;
+    S.xslots = ctx->lean ? S.kmax : simt_split(fp64, 2 * ns, S.Ng, S.kmax, room * S.kmax) * S.kmax;
+    // X'' of a point's k_max directions; lean: of as many as 512 MB hold, for all points
+    ctx->kp_ydirs = S.kmax;
+    if (ctx->lean) ctx->kp_ydirs = (int)std::min<size_t>(S.kmax, std::max<size_t>(1, (512ull << 20) / (mat2 * csz)));
   }
   const int io = o.io_dtype;
   const size_t isz = io == LRDM_DTYPE_F64 ? sizeof(double) : sizeof(float);
   void* stack = nullptr;                       // tensor cores: [N_g][2 N_s] io dtype, set-up only
-  if (tc && cudaMalloc(&stack, npsi * 2 * isz) != cudaSuccess) return LRDM_ERR_OOM;
+  if (tc) LRDM_CK(device_alloc(&stack, npsi * 2 * isz));
   lrdm_status rc = LRDM_OK;
   for (int q = 0; q < nk && rc == LRDM_OK; ++q) {
     rc = [&]() -> lrdm_status {
@@ -301,7 +320,8 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
         LRDM_CU(launch_kp_copy(fp64, in.psi_re[q], io, in.ld_psi, S.Ng, ns, ctx->kp_C[q], 2 * ns, 0, st));
         LRDM_CU(launch_kp_copy(fp64, in.psi_im[q], io, in.ld_psi, S.Ng, ns, ctx->kp_C[q], 2 * ns, ns, st));
         LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_P[q]), S.xslots * mat2 * csz));
-        LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_Y[q]), (size_t)S.kmax * mat2 * csz));
+        if (ctx->lean && q > 0) ctx->kp_Y[q] = ctx->kp_Y[0];
+        else LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&ctx->kp_Y[q]), (size_t)ctx->kp_ydirs * mat2 * csz));
         if (!in.rho)
           LRDM_CU(launch_kp_density(fp64, ctx->kp_C[q], static_cast<const char*>(ctx->kp_C[q]) + ns * csz, ns,
                                     2 * ns, S.Ng, ctx->kp_occ[q], S.g * ctx->kp_w[q], q == 0, in.rho_floor,
@@ -337,7 +357,7 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
       LRDM_CU(cudaStreamSynchronize(st));      // the stacked copy is reused for the next point
       // room for up to 4 grid-row ranges of the projection (kp_choose_split),
       // fewer where that would exceed 1 GB per point
-      int cap = 4;
+      int cap = ctx->lean ? 1 : 4;
       while (cap > 1 && (size_t)cap * S.kmax * ld2 * sizeof(float) > ((size_t)1 << 30)) --cap;
       ctx->kp_split_cap = cap;
       LRDM_CK(dalloc(ctx, reinterpret_cast<char**>(&c.Xpart), (size_t)cap * S.kmax * ld2 * sizeof(float)));
@@ -368,6 +388,47 @@ lrdm_status kp_setup(lrdm_ctx* ctx, const lrdm_kpoint_system& in, cudaStream_t s
     ctx->tc_entries.reserve(nk);
   }
   LRDM_CU(cudaStreamSynchronize(st));   // the host eps / occ vectors end here
+  return LRDM_OK;
+}
+
+// A context of the validated system (lean: with the least memory).
+lrdm_status make_kp_ctx(lrdm_ctx** out, const lrdm_kpoint_system& sys, const lrdm_options& o, void* stream,
+                        bool lean) {
+  lrdm_ctx* ctx = new (std::nothrow) lrdm_ctx();
+  if (!ctx) return LRDM_ERR_OOM;
+  ctx->lean = lean;
+  ctx->nsys = 1;
+  ctx->opt = o;
+  cudaGetDevice(&ctx->device);
+  cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
+  ctx->sys = new (std::nothrow) SysState[1];
+  if (!ctx->sys) {
+    delete ctx;
+    return LRDM_ERR_OOM;
+  }
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  ctx->setup_st = st;
+  lrdm_status rc = LRDM_OK;
+  do {
+    if ((rc = dalloc(ctx, &ctx->d_status, 1)) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->d_round, 1)) != LRDM_OK) break;
+    const int maxval = KMAX_LIMIT * (KMAX_LIMIT + 1) / 2 + KMAX_LIMIT + 1;
+    if ((rc = dalloc(ctx, &ctx->ls_partial, (size_t)LS_BLOCKS * maxval)) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->ls_sums, maxval)) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->ls_coef, KMAX_LIMIT)) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->ls_scal, 4)) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->upd_partial, UPD_BLOCKS)) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->gs_scratch, gram_schmidt_scratch())) != LRDM_OK) break;
+    if ((rc = dalloc(ctx, &ctx->gs_norm, 1)) != LRDM_OK) break;
+    if ((rc = kp_setup(ctx, sys, st)) != LRDM_OK) break;
+    if (is_tc(o.prec) && o.autotune && (rc = autotune(ctx, st)) != LRDM_OK) break;
+    if (cudaGetLastError() != cudaSuccess) rc = LRDM_ERR_CUDA;
+  } while (0);
+  if (rc != LRDM_OK) {
+    free_ctx(ctx);
+    return rc;
+  }
+  *out = ctx;
   return LRDM_OK;
 }
 
@@ -402,41 +463,8 @@ lrdm_status lrdm_kp_create(lrdm_ctx** out, const lrdm_kpoint_system* sys, const 
     return LRDM_ERR_INVALID_ARG;
   if (is_tc(o.prec) && !tc_supported()) return LRDM_ERR_UNSUPPORTED;
   if (!(o.degen_tol >= 0.0) || (o.poisson_symbol != 0 && o.poisson_symbol != 1)) return LRDM_ERR_INVALID_ARG;
-  lrdm_ctx* ctx = new (std::nothrow) lrdm_ctx();
-  if (!ctx) return LRDM_ERR_OOM;
-  ctx->nsys = 1;
-  ctx->opt = o;
-  cudaGetDevice(&ctx->device);
-  cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
-  ctx->sys = new (std::nothrow) SysState[1];
-  if (!ctx->sys) {
-    delete ctx;
-    return LRDM_ERR_OOM;
-  }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  ctx->setup_st = st;
-  lrdm_status rc = LRDM_OK;
-  do {
-    if ((rc = dalloc(ctx, &ctx->d_status, 1)) != LRDM_OK) break;
-    if ((rc = dalloc(ctx, &ctx->d_round, 1)) != LRDM_OK) break;
-    const int maxval = KMAX_LIMIT * (KMAX_LIMIT + 1) / 2 + KMAX_LIMIT + 1;
-    if ((rc = dalloc(ctx, &ctx->ls_partial, (size_t)LS_BLOCKS * maxval)) != LRDM_OK) break;
-    if ((rc = dalloc(ctx, &ctx->ls_sums, maxval)) != LRDM_OK) break;
-    if ((rc = dalloc(ctx, &ctx->ls_coef, KMAX_LIMIT)) != LRDM_OK) break;
-    if ((rc = dalloc(ctx, &ctx->ls_scal, 4)) != LRDM_OK) break;
-    if ((rc = dalloc(ctx, &ctx->upd_partial, UPD_BLOCKS)) != LRDM_OK) break;
-    if ((rc = dalloc(ctx, &ctx->gs_scratch, gram_schmidt_scratch())) != LRDM_OK) break;
-    if ((rc = dalloc(ctx, &ctx->gs_norm, 1)) != LRDM_OK) break;
-    if ((rc = kp_setup(ctx, *sys, st)) != LRDM_OK) break;
-    if (is_tc(o.prec) && o.autotune && (rc = autotune(ctx, st)) != LRDM_OK) break;
-    if (cudaGetLastError() != cudaSuccess) rc = LRDM_ERR_CUDA;
-  } while (0);
-  if (rc != LRDM_OK) {
-    free_ctx(ctx);
-    return rc;
-  }
-  *out = ctx;
-  return LRDM_OK;
+  const lrdm_status rc = make_kp_ctx(out, *sys, o, stream, false);
+  return rc == LRDM_ERR_OOM ? make_kp_ctx(out, *sys, o, stream, true) : rc;
 }
 
 lrdm_status lrdm_kp_get_split(lrdm_ctx* ctx, int K, int* split) {

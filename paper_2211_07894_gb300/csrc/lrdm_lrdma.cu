@@ -40,7 +40,7 @@ namespace {
 template <typename T>
 lrdm_status lalloc(lrdm_lrdma* a, T** p, size_t count) {
   void* q = nullptr;
-  if (cudaMalloc(&q, (count ? count : 1) * sizeof(T)) != cudaSuccess) return LRDM_ERR_OOM;
+  LRDM_CK(device_alloc(&q, (count ? count : 1) * sizeof(T)));
   a->allocs.push_back(q);
   if (cudaMemset(q, 0, (count ? count : 1) * sizeof(T)) != cudaSuccess) return LRDM_ERR_CUDA;
   *p = static_cast<T*>(q);
