@@ -267,7 +267,9 @@ struct DmuArgs {
 // exponential of the distance to mu and leaves the FP32 range where a gap is
 // wide.  FP32 partials of X are added up as FP32 pairs first.  Bound by the
 // latency of its strided loads and by the block's FP64 additions: 512 threads
-// where the partials are FP32 (N_s = 1024, seven ranges: 13 us; 256: 18, 1024: 14).
+// where the partials are FP32 (N_s = 1024, seven ranges: 11.6 us; 256: 18, 1024:
+// 14), and the states one after the other, so that the loads of a state's ranges
+// are in flight together (FP64, 38 ranges: 8.6 us; four states unrolled: 17.5).
 template <typename T>
 constexpr int TRACE_THREADS = sizeof(T) == 8 ? 256 : 512;
 template <typename T>
@@ -276,7 +278,7 @@ __device__ __forceinline__ void trace_sums(const DmuArgs& A, int k, double& num,
   num = den = 0.0;
   for (int s = 0; s < A.nspin; ++s) {
     const long long mat = (long long)A.ldx[s] * A.ldx[s];
-#pragma unroll 4
+#pragma unroll 1
     for (int i = threadIdx.x; i < A.ns[s]; i += blockDim.x) {
       const double x = sum_strided(static_cast<const T*>(A.X[s]) + k * mat + (long long)i * A.ldx[s] + i,
                                    A.nsplit, A.K * mat);

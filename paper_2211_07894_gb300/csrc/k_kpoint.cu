@@ -18,7 +18,8 @@ namespace {
 
 // mu'_k over all k-points: one block per direction over all (point, state)
 // pairs, FP64 sums by as many threads as in trace_sums (k_elem.cu; 48^3, 4
-// points of 512: 12 us, 256 or 1024 threads 13 and 15).
+// points of 512: 12 us, 256 or 1024 threads 13 and 15), the states one after the
+// other.
 template <typename T>
 constexpr int KP_DMU_THREADS = sizeof(T) == 8 ? 256 : 512;
 template <typename T>
@@ -29,7 +30,7 @@ __global__ void __launch_bounds__(KP_DMU_THREADS<T>)
   const int k = blockIdx.x;
   const long long mat = (long long)A.ld * A.ld;
   double num = 0.0, den = 0.0;
-#pragma unroll 4
+#pragma unroll 1
   for (int e = threadIdx.x; e < A.nk * A.ns; e += blockDim.x) {
     const int kp = e / A.ns, i = e - kp * A.ns;
     const double l = A.kw[kp] * A.L[kp][(long long)i * A.ns + i];
