@@ -127,8 +127,7 @@ typedef struct lrdm_options {
                             own problems and keeps the fastest; with the
                             environment variable LRDM_TUNE_CACHE naming a file,
                             results are read from / appended to it (one JSON
-                            object per line, keyed by kernel version, device and
-                            problem sizes) */
+                            object per line, keyed by device and problem sizes) */
   int debug_flags;       /* test-only fault injection, 0 in production:
                             LRDM_DEBUG_STALL_PROJECTION makes the next
                             tensor-core projection launch (once) leave one

@@ -556,14 +556,7 @@ TcEntry tc_entry(lrdm_ctx* ctx, int s, int c, int K) {
 // autotuner: launch shape of the tensor-core contractions
 // ---------------------------------------------------------------------------
 
-// Version of the contraction kernels, part of every cache key: raised whenever
-// their launch shapes time differently, so that a cache file written against
-// other kernels is not read (2: two-direction projection items, the response's
-// triangle).
-constexpr int TUNE_VERSION = 2;
-
-// Identifies the problem set (kernels, device, precision, every (N_g, N_s padded,
-// k_max)).
+// Identifies the problem set (device, precision, every (N_g, N_s padded, k_max)).
 std::string tune_key(lrdm_ctx* ctx) {
   int dev = 0, sms = 0, major = 0, minor = 0;
   cudaGetDevice(&dev);
@@ -571,7 +564,7 @@ std::string tune_key(lrdm_ctx* ctx) {
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
   std::string k = "sm" + std::to_string(major) + std::to_string(minor) + "x" + std::to_string(sms) +
-                  ";prec" + std::to_string(ctx->opt.prec) + ";kernels" + std::to_string(TUNE_VERSION);
+                  ";prec" + std::to_string(ctx->opt.prec);
   if (ctx->kp) {                      // one stacked problem per k-point
     for (const Channel& c : ctx->kp_ch)
       k += ";kp" + std::to_string(ctx->sys[0].Ng) + "," + std::to_string(c.ns_pad) + "," +
