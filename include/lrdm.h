@@ -127,7 +127,8 @@ typedef struct lrdm_options {
                             own problems and keeps the fastest; with the
                             environment variable LRDM_TUNE_CACHE naming a file,
                             results are read from / appended to it (one JSON
-                            object per line, keyed by device and problem sizes) */
+                            object per line, keyed by device and problem sizes;
+                            delete it when the library changes) */
   int debug_flags;       /* test-only fault injection, 0 in production:
                             LRDM_DEBUG_STALL_PROJECTION makes the next
                             tensor-core projection launch (once) leave one
@@ -163,8 +164,11 @@ void lrdm_default_options(lrdm_options* opt);
  * (g sum f(eps, mu) = N_e by FP64 bisection, Eq. kseqcont; spin channels share
  * mu, §II.D), computes the occupations, the Loewner matrices, f_xc, the
  * density if it is not given, the operand copies of Psi for the chosen
- * precision, cuFFT plans and all workspaces.  Synchronises the stream before
- * returning.  On error *out is NULL and nothing is leaked. */
+ * precision, cuFFT plans and all workspaces.  Reads the caller's arrays in the
+ * order of the stream and synchronises it before returning.  Where the device's
+ * memory does not hold the workspaces that only buy speed (partial projections of
+ * several row ranges), the context is made without them.  On error *out is NULL
+ * and nothing is leaked. */
 lrdm_status lrdm_create(lrdm_ctx** out, const lrdm_system* sys, int nsys,
                         const lrdm_options* opt, void* stream);
 
@@ -468,7 +472,8 @@ typedef struct lrdm_kpoint_system {
 /* Creates a context for one Brillouin-zone-sampled system: copies each Psi
  * plane into the compute type (the caller's buffers are not kept), solves mu
  * over all k-points on the host, builds the Loewner matrices, the density if
- * not given, f_x and the Poisson plans.  Synchronises the stream.
+ * not given, f_x and the Poisson plans.  Synchronises the stream; short of memory
+ * as lrdm_create.
  * Errors: INVALID_ARG (null pointers, nk outside 1..32, weights not positive
  * or not summing to 1, kT <= 0, bad options), MU_NOT_CONVERGED (N_e outside
  * what the states can hold), UNSUPPORTED (tensor-core precision on a device

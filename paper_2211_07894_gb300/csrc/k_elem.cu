@@ -425,7 +425,8 @@ __global__ void __launch_bounds__(TRACE_THREADS<T>) k_trace_bar(DmuArgs A, doubl
 // so the directions of a row are shared out where threads are left over, and
 // the diagonal's FP64 sums are one direction a lane: 48^3, N_s = 512, K = 8,
 // seven row ranges: 116 -> 32 us (one thread summed the diagonal, 56 terms one
-// after the other).  Four blocks an SM: with two the FP32 form took 41 us.
+// after the other).  Four blocks an SM, although the FP32 form then spills 324
+// bytes a thread: 31.7 us, with three blocks (24 bytes) 46, with two 40.5.
 //
 // With FP32 partials (the tensor-core and FP32 modes) Lbar_ij (j != i) is
 // summed over the directions in FP32, four consecutive j per thread with
